@@ -78,7 +78,7 @@ struct ges_scene {
     int device = 0;
     cudaStream_t stream = nullptr;
     DevBuf s_rec, s_rgb, g_rec, s_vis, g_vis;
-    DevBuf s_cnt, g_cnt, s_off, g_off, s_cur, g_cur;
+    DevBuf s_cnt, g_cnt, s_rng, g_rng;
     DevBuf s_list, g_list;
     DevBuf hist, base, vcount;     // local binning
     DevBuf status;                 // ST_WORDS per view slot
@@ -229,19 +229,18 @@ ges_status ensure_scratch(ges_scene *s, int64_t T, int slots, cudaStream_t st)
             if ((e = b->ensure((Tc + 1) * 4))) return cuda_fail(e, "scratch allocation (tile counts)");
             if ((e = cudaMemsetAsync(b->p, 0, (Tc + 1) * 4, st))) return cuda_fail(e, "cudaMemsetAsync");
         }
-        if ((e = s->s_off.ensure((Tc + 1) * 4)) || (e = s->g_off.ensure((Tc + 1) * 4)) ||
-            (e = s->s_cur.ensure((Tc + 1) * 4)) || (e = s->g_cur.ensure((Tc + 1) * 4)))
-            return cuda_fail(e, "scratch allocation (tile offsets)");
+        if ((e = s->s_rng.ensure(Tc * 8)) || (e = s->g_rng.ensure(Tc * 8)))
+            return cuda_fail(e, "scratch allocation (tile ranges)");
         s->tiles_cap = Tc;
     }
     {
-        // local binning: one histogram row and one base row per preprocess CTA
+        // local binning: one histogram row and one row of list starts per preprocess CTA
         int sms = 152;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s->device);
         const LocalBins B = plan_local_bins(s->desc.n_surfels, s->desc.n_gaussians, sms);
         const int64_t P = std::max(B.Ps + B.Pg, 1), Tl = std::min<int64_t>(T, kLocalMaxTiles);
-        if ((e = s->hist.ensure((size_t)P * ((Tl + 1) / 2) * 4)) || (e = s->base.ensure((size_t)P * Tl * 4)) ||
-            (e = s->vcount.ensure((size_t)P * 4)))
+        const size_t row = (size_t)((Tl + 1) / 2) * 4;   // packed pairs of tiles
+        if ((e = s->hist.ensure(P * row)) || (e = s->base.ensure(2 * P * row)) || (e = s->vcount.ensure((size_t)P * 4)))
             return cuda_fail(e, "scratch allocation (bins)");
     }
     if (s->s_cap == 0) s->s_cap = std::max<int64_t>((int64_t)1 << 20, 4 * s->desc.n_surfels);
@@ -264,8 +263,7 @@ ViewScratch scratch_of(ges_scene *s, int slot)
     X.s_rec = (float4 *)s->s_rec.p; X.s_rgb = (float4 *)s->s_rgb.p; X.g_rec = (float4 *)s->g_rec.p;
     X.s_vis = (int *)s->s_vis.p; X.g_vis = (int *)s->g_vis.p;
     X.s_cnt = (int *)s->s_cnt.p; X.g_cnt = (int *)s->g_cnt.p;
-    X.s_off = (int *)s->s_off.p; X.g_off = (int *)s->g_off.p;
-    X.s_cur = (int *)s->s_cur.p; X.g_cur = (int *)s->g_cur.p;
+    X.s_rng = (int2 *)s->s_rng.p; X.g_rng = (int2 *)s->g_rng.p;
     X.s_list = (int *)s->s_list.p; X.g_list = (int *)s->g_list.p;
     X.s_cap = s->s_cap; X.g_cap = s->g_cap;
     X.status = (unsigned *)s->status.p + (size_t)slot * ST_WORDS;
@@ -434,9 +432,9 @@ ges_status ges_destroy_scene(ges_scene *s)
 {
     if (!s) return GES_OK;
     cudaStreamSynchronize(s->stream);
-    DevBuf *bufs[] = {&s->s_rec, &s->s_rgb, &s->g_rec, &s->s_vis, &s->g_vis, &s->s_cnt, &s->g_cnt, &s->s_off,
-                      &s->g_off, &s->s_cur, &s->g_cur, &s->s_list, &s->g_list, &s->hist, &s->base,
-                      &s->vcount, &s->status, &s->filt, &s->g_aux, &s->t_side, &s->t_keys, &s->t_acc};
+    DevBuf *bufs[] = {&s->s_rec, &s->s_rgb, &s->g_rec, &s->s_vis, &s->g_vis, &s->s_cnt, &s->g_cnt, &s->s_rng,
+                      &s->g_rng, &s->s_list, &s->g_list, &s->hist, &s->base, &s->vcount,
+                       &s->status, &s->filt, &s->g_aux, &s->t_side, &s->t_keys, &s->t_acc};
     for (DevBuf *b : bufs) b->release();
     if (s->bcache) batch_release(s->bcache);
     if (s->status_host) cudaFreeHost(s->status_host);
@@ -833,25 +831,22 @@ size_t batch_layout(ges_batch *b, const std::vector<SceneView> &S, const std::ve
         prep_base += B.Ps + B.Pg;
         sprep_base += B.Ps;
         gprep_base += B.Pg;
-        col_base += (T + 31) / 32;
+        col_base += (T + kColTiles - 1) / kColTiles;
         ViewScratch &X = bv.X;
         X.s_rec = (float4 *)take(N * 64);
         X.s_rgb = (float4 *)take(N * 16);
         X.g_rec = (float4 *)take(M * 64);
         X.s_vis = (int *)take(N * 16);   // 16-byte segment entries (local bins)
         X.g_vis = (int *)take(M * 16);
-        X.s_cnt = (int *)take((T + 1) * 4);
-        X.g_cnt = (int *)take((T + 1) * 4);
-        X.s_off = (int *)take((T + 1) * 4);
-        X.g_off = (int *)take((T + 1) * 4);
-        X.s_cur = (int *)take((T + 1) * 4);
-        X.g_cur = (int *)take((T + 1) * 4);
+        X.s_cnt = X.g_cnt = nullptr;     // atomic binning only
+        X.s_rng = (int2 *)take((size_t)T * 8);
+        X.g_rng = (int2 *)take((size_t)T * 8);
         X.s_cap = b->s_cap[v];
         X.g_cap = b->g_cap[v];
         X.s_list = (int *)take(b->s_cap[v] * 4);
         X.g_list = (int *)take(b->g_cap[v] * 4);
         X.hist = (unsigned *)take((size_t)P * ((T + 1) / 2) * 4);
-        X.base = (unsigned *)take((size_t)P * T * 4);
+        X.base = (unsigned *)take((size_t)P * ((T + 1) / 2) * 8);
         X.vcount = (unsigned *)take((size_t)P * 4);
         X.g_aux = S[v].gdim == 2 ? (float4 *)take(M * 32) : nullptr;
         X.g_col = (float4 *)take(M * 16);
@@ -1149,7 +1144,7 @@ static ges_status batch_create(ges_scene *const *scenes, const ges_camera *cams,
                 P.total_prep += b->views[v].B.Ps + b->views[v].B.Pg;
                 P.total_sprep += b->views[v].B.Ps;
                 P.total_gprep += b->views[v].B.Pg;
-                P.total_colscan += (b->views[v].T + 31) / 32;
+                P.total_colscan += (b->views[v].T + kColTiles - 1) / kColTiles;
                 P.max_T = std::max(P.max_T, b->views[v].T);
             }
             std::memcpy(b->h_table, b->views.data(), sizeof(BatchView) * n_views);
@@ -1462,14 +1457,12 @@ constexpr size_t kNaSRgb = na_align(kNaSRec + kNaMaxSurfels * 64);
 constexpr size_t kNaGRec = na_align(kNaSRgb + kNaMaxSurfels * 16);
 constexpr size_t kNaSVis = na_align(kNaGRec + kNaMaxGaussians * 64);
 constexpr size_t kNaGVis = na_align(kNaSVis + kNaMaxSurfels * 4);
-constexpr size_t kNaTileBytes = na_align((kNaMaxTiles + 1) * 4);
+constexpr size_t kNaTileBytes = na_align(kNaMaxTiles * 4);
 constexpr size_t kNaSCnt = na_align(kNaGVis + kNaMaxGaussians * 4);   // s_cnt, g_cnt adjacent (cleared together)
 constexpr size_t kNaGCnt = kNaSCnt + kNaTileBytes;
-constexpr size_t kNaSOff = kNaGCnt + kNaTileBytes;
-constexpr size_t kNaGOff = kNaSOff + kNaTileBytes;
-constexpr size_t kNaSCur = kNaGOff + kNaTileBytes;
-constexpr size_t kNaGCur = kNaSCur + kNaTileBytes;
-constexpr size_t kNaStatus = kNaGCur + kNaTileBytes;
+constexpr size_t kNaSRng = kNaGCnt + kNaTileBytes;
+constexpr size_t kNaGRng = kNaSRng + 2 * kNaTileBytes;
+constexpr size_t kNaStatus = kNaGRng + 2 * kNaTileBytes;
 constexpr size_t kNaSList = na_align(kNaStatus + ST_WORDS * 4);
 constexpr size_t kNaGList = na_align(kNaSList + kNaMaxPairs * 4);
 constexpr size_t kNaBytes = na_align(kNaGList + kNaMaxPairs * 4);
@@ -1531,8 +1524,7 @@ extern "C" GES_API ges_status ges_render_noalloc(const ges_scene_desc *desc, con
     X.s_rec = (float4 *)(base + kNaSRec); X.s_rgb = (float4 *)(base + kNaSRgb); X.g_rec = (float4 *)(base + kNaGRec);
     X.s_vis = (int *)(base + kNaSVis); X.g_vis = (int *)(base + kNaGVis);
     X.s_cnt = (int *)(base + kNaSCnt); X.g_cnt = (int *)(base + kNaGCnt);
-    X.s_off = (int *)(base + kNaSOff); X.g_off = (int *)(base + kNaGOff);
-    X.s_cur = (int *)(base + kNaSCur); X.g_cur = (int *)(base + kNaGCur);
+    X.s_rng = (int2 *)(base + kNaSRng); X.g_rng = (int2 *)(base + kNaGRng);
     X.s_list = (int *)(base + kNaSList); X.g_list = (int *)(base + kNaGList);
     X.s_cap = kNaMaxPairs; X.g_cap = kNaMaxPairs;
     X.status = (unsigned *)(base + kNaStatus);

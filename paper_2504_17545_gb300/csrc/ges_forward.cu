@@ -8,8 +8,8 @@
 //                 counts tile overlaps in a shared-memory histogram (16-bit
 //                 counters packed in pairs), which it writes out as one row.
 //   k_colscan     per tile, exclusive scan of those rows over the CTAs (each
-//                 CTA's start inside the tile's list) and the tile total.
-//   k_scan        exclusive scan of the tile totals, capacity check.
+//                 CTA's start inside the tile's list), the place of the tile's
+//                 list, and the capacity check.
 //   k_fill_local  each CTA re-walks its visible segment and places every
 //                 (tile, primitive) pair with shared-memory cursors.
 //   k_raster      one CTA per 16x16 tile: the CTA stages 256 records at a time
@@ -18,7 +18,10 @@
 //                 lexicographic min of (depth, surfel id); pass 2 accumulates
 //                 the depth-tested Gaussians (Eq. 2-4); the epilogue applies
 //                 Eq. 5.  Everything per pixel stays in registers.
-// No global atomics are needed for binning, so hot tiles do not serialise.
+// No global atomics per primitive are needed for binning, so hot tiles do not
+// serialise.  (Histogram counts added to global per-tile totals by each
+// preprocess CTA, instead of rows and a column scan, cost 97 us of a 4K view's
+// preprocess and 5 us of every view of a batch.)
 // Very large images (more than 32768 tiles) and callers without binning
 // scratch use k_prep_atomic / k_fill_atomic instead (global counters).
 //
@@ -218,46 +221,95 @@ __global__ void __launch_bounds__(kPrepThreads, 2) k_prep_local(SceneView S, Cam
     prep_local_body<kGd, kTr>(S, C, O, X, B, blockIdx.x, hist, vcnt);
 }
 
-__device__ __forceinline__ unsigned hist_get(const unsigned *row, int t)
+// Space for the lists of the tiles whose totals a warp holds (n tiles on each
+// lane, their sum in tot): one addition to the list space handed out so far,
+// so the lists lie in the order the warps arrive in (nothing depends on it).
+// Returns the start of the lane's first list.
+__device__ __forceinline__ int alloc_lists(const ViewScratch &X, bool surf, int64_t tot)
 {
-    const unsigned w = row[t >> 1];
-    return (t & 1) ? (w >> 16) : (w & 0xffffu);
+    const int lane = (int)lane_id();
+    int64_t incl = tot;                  // 64 bits: lists too large are found, not wrapped
+    for (int d = 1; d < 32; d <<= 1) {
+        const int64_t y = __shfl_up_sync(0xffffffffu, incl, d);
+        if (lane >= d) incl += y;
+    }
+    int64_t at = 0;
+    if (lane == 31) {
+        unsigned long long *space = reinterpret_cast<unsigned long long *>(X.status + (surf ? ST_SCUR : ST_GCUR));
+        at = (int64_t)atomicAdd(space, (unsigned long long)incl);
+        atomicAdd(X.status + (surf ? ST_SPAIRS : ST_GPAIRS), (unsigned)incl);
+        if (at + incl > (surf ? X.s_cap : X.g_cap)) atomicOr(X.status + ST_FLAGS, surf ? FLAG_SOVF : FLAG_GOVF);
+    }
+    return (int)(__shfl_sync(0xffffffffu, at, 31) + incl - tot);
 }
 
-// Per tile: exclusive scan over the CTAs of one kind.  Block = 32 tiles x 8
-// warps; warp w scans CTAs [w*P/8, (w+1)*P/8).
+// Per tile: exclusive scan of the counts over the CTAs of one kind, and a
+// place for the tile's list.  Block = 64 tiles x kW warps: a lane takes one
+// histogram word (two tiles), warp w the CTAs [w P/kW, (w+1) P/kW).  A single
+// view is bound by the latency of the rows' loads, so 32 warps share the CTAs
+// of a tile there; in a batch the blocks of the other views hide it, and 8
+// warps have fewer barriers and partial sums per row.  Scanning the totals in
+// a launch of its own, by one CTA per kind, the two launches took 27.9 us of a
+// 1080p view (1M + 300k primitives) and 115.5 us of a 4K one (2.25M + 750k);
+// this one takes 10.8 and 23.1 us.
+template <int kW>
 __device__ __forceinline__ void colscan_body(const ViewScratch &X, int T, const LocalBins &B, int bx, bool surf,
-                                             unsigned (*part)[33])
+                                             unsigned (*part)[kColTiles + 1])
 {
     const int P = surf ? B.Ps : B.Pg, r0 = surf ? 0 : B.Ps;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int t = bx * 32 + lane;
-    const int words = (T + 1) >> 1;
-    const int a = r0 + (int)((int64_t)P * w / 8), b = r0 + (int)((int64_t)P * (w + 1) / 8);
-    unsigned s = 0;
-    if (t < T)
-        for (int r = a; r < b; ++r) s += hist_get(X.hist + (size_t)r * words, t);
-    part[w][lane] = s;
-    __syncthreads();
-    unsigned pre = 0, tot = 0;
-    for (int k = 0; k < 8; ++k) {
-        const unsigned v = part[k][lane];
-        if (k < w) pre += v;
-        tot += v;
-    }
-    if (t < T) {
+    const int words = (T + 1) >> 1, word = bx * 32 + lane;
+    const int a = r0 + (int)((int64_t)P * w / kW), b = r0 + (int)((int64_t)P * (w + 1) / kW);
+    const unsigned *h = X.hist + word;
+    unsigned s0 = 0, s1 = 0;
+    if (word < words) {
+#pragma unroll 8
         for (int r = a; r < b; ++r) {
-            X.base[(size_t)r * T + t] = pre;
-            pre += hist_get(X.hist + (size_t)r * words, t);
+            const unsigned v = h[(size_t)r * words];
+            s0 += v & 0xffffu;
+            s1 += v >> 16;
         }
-        if (w == 0) (surf ? X.s_cnt : X.g_cnt)[t] = (int)tot;
+    }
+    part[w][2 * lane] = s0;
+    part[w][2 * lane + 1] = s1;
+    __syncthreads();
+    // the warps' sums of each tile in turn (row kW: the totals); groups of kW
+    // lanes, one tile each
+    for (int q = threadIdx.x / kW; q < kColTiles; q += 32) {
+        const int k = threadIdx.x % kW;
+        const unsigned v = part[k][q];
+        unsigned incl = v;
+        for (int d = 1; d < kW; d <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, incl, d, kW);
+            if (k >= d) incl += y;
+        }
+        part[k][q] = incl - v;
+        if (k == kW - 1) part[kW][q] = incl;
+    }
+    __syncthreads();
+    if (w == 0) {
+        const int n0 = (int)part[kW][2 * lane], n1 = (int)part[kW][2 * lane + 1];
+        const int at = alloc_lists(X, surf, (int64_t)n0 + n1);
+        int2 *rng = surf ? X.s_rng : X.g_rng;
+        if (2 * word < T) rng[2 * word] = make_int2(at, at + n0);
+        if (2 * word + 1 < T) rng[2 * word + 1] = make_int2(at + n0, at + n0 + n1);
+    }
+    if (word >= words) return;
+    unsigned p0 = part[w][2 * lane], p1 = part[w][2 * lane + 1];
+    uint2 *out = reinterpret_cast<uint2 *>(X.base) + word;
+#pragma unroll 8
+    for (int r = a; r < b; ++r) {
+        const unsigned v = h[(size_t)r * words];
+        out[(size_t)r * words] = make_uint2(p0, p1);
+        p0 += v & 0xffffu;
+        p1 += v >> 16;
     }
 }
 
-__global__ void __launch_bounds__(256) k_colscan(ViewScratch X, int T, LocalBins B)
+__global__ void __launch_bounds__(1024) k_colscan(ViewScratch X, int T, LocalBins B)
 {
-    __shared__ unsigned part[8][33];
-    colscan_body(X, T, B, blockIdx.x, blockIdx.y == 0, part);
+    __shared__ unsigned part[33][kColTiles + 1];
+    colscan_body<32>(X, T, B, blockIdx.x, blockIdx.y == 0, part);
 }
 
 __device__ __forceinline__ void fill_local_body(const ViewScratch &X, int T, int tiles_x, int tsx, int tsy,
@@ -265,9 +317,9 @@ __device__ __forceinline__ void fill_local_body(const ViewScratch &X, int T, int
 {
     if (X.status[ST_FLAGS] & (FLAG_SOVF | FLAG_GOVF)) return;
     const bool surf = c < B.Ps;
-    const int *off = surf ? X.s_off : X.g_off;
-    const unsigned *brow = X.base + (size_t)c * T;
-    for (int t = threadIdx.x; t < T; t += kFillThreads) cur[t] = (unsigned)off[t] + brow[t];
+    const int2 *rng = surf ? X.s_rng : X.g_rng;
+    const unsigned *brow = X.base + (size_t)c * (2 * ((T + 1) >> 1));
+    for (int t = threadIdx.x; t < T; t += kFillThreads) cur[t] = (unsigned)rng[t].x + brow[t];
     __syncthreads();
     const int64_t beg = (int64_t)(surf ? c : c - B.Ps) * (surf ? B.Rs : B.Rg);
     const int4 *seg = reinterpret_cast<const int4 *>(surf ? X.s_vis : X.g_vis) + beg;
@@ -322,13 +374,13 @@ __global__ void __launch_bounds__(256) k_prep_atomic(SceneView S, CamParams C, O
     append_visible(vis, i, X.status + (surf ? ST_SVIS : ST_GVIS), surf ? X.s_vis : X.g_vis);
 }
 
-__device__ __forceinline__ void fill_one(const float4 *rec, int id, int tiles_x, int tsx, int tsy, int *cur, int *list)
+__device__ __forceinline__ void fill_one(const float4 *rec, int id, int tiles_x, int tsx, int tsy, int2 *rng, int *list)
 {
     const float4 r3 = rec[4 * (int64_t)id + 3];
     const unsigned lo = __float_as_uint(r3.y), hi = __float_as_uint(r3.z);
     const int x0 = lo & 0xffff, y0 = lo >> 16, x1 = hi & 0xffff, y1 = hi >> 16;
     for (int ty = y0 >> tsy; ty <= y1 >> tsy; ++ty)
-        for (int tx = x0 >> tsx; tx <= x1 >> tsx; ++tx) list[atomicAdd(cur + ty * tiles_x + tx, 1)] = id;
+        for (int tx = x0 >> tsx; tx <= x1 >> tsx; ++tx) list[atomicAdd(&rng[ty * tiles_x + tx].y, 1)] = id;
 }
 
 __global__ void __launch_bounds__(256) k_fill_atomic(ViewScratch X, int tiles_x, int tsx, int tsy)
@@ -337,59 +389,26 @@ __global__ void __launch_bounds__(256) k_fill_atomic(ViewScratch X, int tiles_x,
     const unsigned ns = X.status[ST_SVIS], ng = X.status[ST_GVIS];
     const unsigned stride = gridDim.x * blockDim.x;
     for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < ns + ng; k += stride) {
-        if (k < ns) fill_one(X.s_rec, X.s_vis[k], tiles_x, tsx, tsy, X.s_cur, X.s_list);
-        else fill_one(X.g_rec, X.g_vis[k - ns], tiles_x, tsx, tsy, X.g_cur, X.g_list);
+        if (k < ns) fill_one(X.s_rec, X.s_vis[k], tiles_x, tsx, tsy, X.s_rng, X.s_list);
+        else fill_one(X.g_rec, X.g_vis[k - ns], tiles_x, tsx, tsy, X.g_rng, X.g_list);
     }
 }
 
 // ---------------------------------------------------------------------------
-// scan of tile totals (both binning modes)
+// list allocation (atomic binning; k_colscan does it for local bins)
 
-__device__ __forceinline__ void scan_body(const ViewScratch &X, int T, bool surf, long long *warp_tot)
+// Places for the lists from the tiles' totals.  The ends start at the lists'
+// starts (the fill moves them), and the counters go back to zero.
+__global__ void __launch_bounds__(kAllocTiles) k_alloc(ViewScratch X, int T)
 {
+    const bool surf = blockIdx.y == 0;
     int *cnt = surf ? X.s_cnt : X.g_cnt;
-    int *off = surf ? X.s_off : X.g_off;
-    int *cur = surf ? X.s_cur : X.g_cur;
-    const int64_t cap = surf ? X.s_cap : X.g_cap;
-    const int tid = threadIdx.x, per = (T + 1023) / 1024;
-    const int b = min(tid * per, T), e = min(b + per, T);
-    long long local = 0;
-    for (int t = b; t < e; ++t) local += cnt[t];
-    long long incl = local;
-    for (int d = 1; d < 32; d <<= 1) {
-        long long y = __shfl_up_sync(0xffffffffu, incl, d);
-        if ((tid & 31) >= d) incl += y;
-    }
-    if ((tid & 31) == 31) warp_tot[tid >> 5] = incl;
-    __syncthreads();
-    if (tid < 32) {
-        long long w = warp_tot[tid], wi = w;
-        for (int d = 1; d < 32; d <<= 1) {
-            long long y = __shfl_up_sync(0xffffffffu, wi, d);
-            if (tid >= d) wi += y;
-        }
-        warp_tot[tid] = wi - w;
-    }
-    __syncthreads();
-    long long run = warp_tot[tid >> 5] + incl - local;
-    for (int t = b; t < e; ++t) {
-        const int c = cnt[t];
-        off[t] = (int)run;
-        cur[t] = (int)run;
+    const int t = blockIdx.x * kAllocTiles + threadIdx.x;
+    const int at = alloc_lists(X, surf, t < T ? cnt[t] : 0);
+    if (t < T) {
+        (surf ? X.s_rng : X.g_rng)[t] = make_int2(at, at);
         cnt[t] = 0;
-        run += c;
     }
-    if (tid == 1023) {
-        off[T] = (int)run;
-        X.status[surf ? ST_SPAIRS : ST_GPAIRS] = (unsigned)run;
-        if (run > cap) atomicOr(X.status + ST_FLAGS, surf ? FLAG_SOVF : FLAG_GOVF);
-    }
-}
-
-__global__ void __launch_bounds__(1024) k_scan(ViewScratch X, int T)
-{
-    __shared__ long long warp_tot[32];
-    scan_body(X, T, blockIdx.x == 0, warp_tot);
 }
 
 // ---------------------------------------------------------------------------
@@ -727,8 +746,8 @@ __device__ __forceinline__ void raster_tile(const ViewScratch &X, const CamParam
     const unsigned warp = threadIdx.x >> 5, lane = lane_id();
     const WarpBlock<kS> B(C, tile, warp, lane);
     const bool do_s = O.mode != GES_MODE_GAUSSIANS_ONLY, do_g = O.mode != GES_MODE_SURFELS_ONLY;
-    const int s0 = do_s ? X.s_off[tile] : 0, s1 = do_s ? X.s_off[tile + 1] : 0;
-    const int g0 = do_g ? X.g_off[tile] : 0, g1 = do_g ? X.g_off[tile + 1] : 0;
+    const int2 sr = do_s ? X.s_rng[tile] : make_int2(0, 0), gr = do_g ? X.g_rng[tile] : make_int2(0, 0);
+    const int s0 = sr.x, s1 = sr.y, g0 = gr.x, g1 = gr.y;
     const int t = threadIdx.x;
 
     // first chunk of both lists together: one round trip, one barrier
@@ -901,7 +920,7 @@ __global__ void __launch_bounds__(kColourThreads) k_bcolour(const BatchView *V, 
 
 __global__ void __launch_bounds__(256) k_bcolscan(const BatchView *V, int n)
 {
-    __shared__ unsigned part[8][33];
+    __shared__ unsigned part[9][kColTiles + 1];
     __shared__ __align__(16) unsigned char bv_raw[sizeof(BatchView)];
     BatchView &bv = *reinterpret_cast<BatchView *>(bv_raw);
     __shared__ int sv;
@@ -909,17 +928,7 @@ __global__ void __launch_bounds__(256) k_bcolscan(const BatchView *V, int n)
     __syncthreads();
     load_view(V, sv, bv);
     __syncthreads();
-    colscan_body(bv.X, bv.T, bv.B, blockIdx.x - bv.colscan_base, blockIdx.y == 0, part);
-}
-
-__global__ void __launch_bounds__(1024) k_bscan(const BatchView *V)
-{
-    __shared__ long long warp_tot[32];
-    __shared__ __align__(16) unsigned char bv_raw[sizeof(BatchView)];
-    BatchView &bv = *reinterpret_cast<BatchView *>(bv_raw);
-    load_view(V, blockIdx.x >> 1, bv);
-    __syncthreads();
-    scan_body(bv.X, bv.T, (blockIdx.x & 1) == 0, warp_tot);
+    colscan_body<8>(bv.X, bv.T, bv.B, blockIdx.x - bv.colscan_base, blockIdx.y == 0, part);
 }
 
 __global__ void __launch_bounds__(kFillThreads) k_bfill(const BatchView *V, int n)
@@ -1015,8 +1024,7 @@ cudaError_t launch_batch(const BatchView *d_views, const BatchPlan &P, const Opt
         }
     }
     mark(1);
-    if (P.total_colscan > 0) k_bcolscan<<<dim3(P.total_colscan, 2), 256, 0, st>>>(d_views, P.n);
-    k_bscan<<<2 * P.n, 1024, 0, st>>>(d_views);
+    k_bcolscan<<<dim3(P.total_colscan, 2), 256, 0, st>>>(d_views, P.n);
     mark(2);
     if (P.total_prep > 0)
         k_bfill<<<P.total_prep, kFillThreads, local_bins_smem(P.max_T, true), st>>>(d_views, P.n);
@@ -1095,8 +1103,8 @@ cudaError_t launch_binning(const SceneView &S, const CamParams &C, const OptPara
         }
     }
     if (ev) cudaEventRecord(ev[1], st);
-    if (local && B.Ps + B.Pg > 0) k_colscan<<<dim3((T + 31) / 32, 2), 256, 0, st>>>(X, T, B);
-    k_scan<<<2, 1024, 0, st>>>(X, T);
+    if (local) k_colscan<<<dim3((T + kColTiles - 1) / kColTiles, 2), 1024, 0, st>>>(X, T, B);
+    else k_alloc<<<dim3((T + kAllocTiles - 1) / kAllocTiles, 2), kAllocTiles, 0, st>>>(X, T);
     if (ev) cudaEventRecord(ev[2], st);
     if (local) {
         if (B.Ps + B.Pg > 0) k_fill_local<<<B.Ps + B.Pg, kFillThreads, local_bins_smem(T, true), st>>>(X, T, C.tiles_x, C.tsx, C.tsy, B);
@@ -1125,10 +1133,10 @@ __global__ void __launch_bounds__(256) k_count(SceneView S, ViewScratch X, CamPa
     for (int kind = 0; kind < 2; ++kind) {
         if (kind == 0 && O.mode == GES_MODE_GAUSSIANS_ONLY) continue;
         if (kind == 1 && O.mode == GES_MODE_SURFELS_ONLY) continue;
-        const int *off = kind == 0 ? X.s_off : X.g_off;
+        const int2 rng = (kind == 0 ? X.s_rng : X.g_rng)[tile];
         const int *list = kind == 0 ? X.s_list : X.g_list;
         const float4 *rec = kind == 0 ? X.s_rec : X.g_rec;
-        const int a = off[tile], b = off[tile + 1];
+        const int a = rng.x, b = rng.y;
         for (int base = a; base < b; base += 256) {
             __syncthreads();
             if (base + t < b) stage_rec(st, rec, list[base + t], t);

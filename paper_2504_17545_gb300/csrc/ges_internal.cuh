@@ -33,6 +33,8 @@ enum : int {
     ST_GFRAG = 6,         // Gaussian pixel terms with alpha >= alpha_min (work count)
     ST_RETIRED = 7,       // batch raster: tiles of this view finished
     ST_TDONE = 8,         // batch raster: %globaltimer (ns, 64-bit, words 8-9) when the last tile finished
+    ST_SCUR = 10,         // tile-list space handed out, surfels (64-bit, words 10-11)
+    ST_GCUR = 12,         // the same for the Gaussians (words 12-13)
     ST_WORDS = 16,
 };
 enum : unsigned { FLAG_SOVF = 1u, FLAG_GOVF = 2u, FLAG_BADQ = 4u };
@@ -77,16 +79,15 @@ struct ViewScratch {
     // (id, bbox lo, bbox hi, -), 16 B per primitive; with atomic binning one
     // id per entry
     int *s_vis, *g_vis;
-    int *s_cnt, *g_cnt;   // [T]     per-tile counts (zero between renders)
-    int *s_off, *g_off;   // [T+1]   exclusive offsets
-    int *s_cur, *g_cur;   // [T]     fill cursors (atomic binning)
+    int *s_cnt, *g_cnt;   // [T]     per-tile counts (atomic binning; zero between renders)
+    int2 *s_rng, *g_rng;  // [T]     (start, end) of each tile's list
     int *s_list, *g_list; // tile lists
     int64_t s_cap, g_cap; // list capacities (entries)
     unsigned *status;     // [ST_WORDS]
     // local binning (per-CTA primitive ranges with shared-memory histograms);
     // left null, the render bins with global atomics instead
     unsigned *hist = nullptr;    // [P][ceil(T/2)] packed 16-bit per-CTA tile counts
-    unsigned *base = nullptr;    // [P][T] per-CTA start inside each tile's list
+    unsigned *base = nullptr;    // [P][2 ceil(T/2)] per-CTA start inside each tile's list
     unsigned *vcount = nullptr;  // [P] visible primitives per CTA
     // [M][2] side data of each Gaussian, written when the render needs it:
     // 2D Gaussians (rgb, log2 sigma'), (normal, log2(alpha_min / sigma'));
@@ -149,6 +150,8 @@ cudaError_t launch_batch(const BatchView *d_views, const BatchPlan &P, const Opt
 LocalBins plan_local_bins_per_cta(int64_t N, int64_t M, int64_t prims_per_cta);
 constexpr int kPrepThreads = 512;
 constexpr int kFillThreads = 1024;
+constexpr int kAllocTiles = 1024;       // tiles per CTA of the list allocation (atomic binning)
+constexpr int kColTiles = 64;           // tiles per CTA of the column scan
 LocalBins plan_local_bins(int64_t N, int64_t M, int num_sms);
 size_t local_bins_smem(int T, bool fill);
 cudaError_t prepare_forward_kernels();   // once per device: large dynamic shared memory

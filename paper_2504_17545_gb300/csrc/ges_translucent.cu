@@ -43,12 +43,12 @@ __device__ __forceinline__ unsigned depth_key(float z)
     return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
 }
 
-__global__ void __launch_bounds__(256) k_tkeys(const int *__restrict__ list, const int *__restrict__ n_ptr,
+__global__ void __launch_bounds__(256) k_tkeys(const int *__restrict__ list,
                                                const float4 *__restrict__ tside, unsigned long long *keys,
                                                const unsigned *status)
 {
     if (status[ST_FLAGS] & FLAG_SOVF) return;     // lists not filled; the count exceeds the capacity
-    const int n = *n_ptr;
+    const int n = (int)status[ST_SPAIRS];
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const int id = list[i];
         keys[i] = ((unsigned long long)depth_key(tside[4 * (int64_t)id].z) << 32) | (unsigned)id;
@@ -79,12 +79,12 @@ __device__ __forceinline__ void bitonic(unsigned long long *a, int n, int m)
     }
 }
 
-__global__ void __launch_bounds__(256) k_tsort(const int *__restrict__ off, unsigned long long *keys, int *list,
+__global__ void __launch_bounds__(256) k_tsort(const int2 *__restrict__ rng, unsigned long long *keys, int *list,
                                                const unsigned *status)
 {
     __shared__ unsigned long long sk[kSortCap];
     if (status[ST_FLAGS] & FLAG_SOVF) return;
-    const int a = off[blockIdx.x], n = off[blockIdx.x + 1] - a;
+    const int a = rng[blockIdx.x].x, n = rng[blockIdx.x].y - a;
     if (n <= 1) return;
     int m = 1;
     while (m < n) m <<= 1;
@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(kRasterThreads, 4)
     const int px = wx0 + (int)(lane & 7), py = wy0 + (int)(lane >> 3);
     const bool in_img = px < C.W && py < C.H;
     const float u = px + 0.5f, v = py + 0.5f;
-    const int s0 = X.s_off[tile], s1 = X.s_off[tile + 1];
+    const int s0 = X.s_rng[tile].x, s1 = X.s_rng[tile].y;
     const int t = threadIdx.x;
     auto stage = [&](int base) {
         if (base + t < s1) {
@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(kRasterThreads, 3)
     const int px = wx0 + (int)(lane & 7), py = wy0 + (int)(lane >> 3);
     const bool in_img = px < C.W && py < C.H;
     const float u = px + 0.5f, v = py + 0.5f;
-    const int s0 = X.s_off[tile], s1 = X.s_off[tile + 1];
+    const int s0 = X.s_rng[tile].x, s1 = X.s_rng[tile].y;
     const int t = threadIdx.x;
     const int64_t HW = (int64_t)C.W * C.H, pix = in_img ? (int64_t)py * C.W + px : 0;
     float g[3] = {0.f, 0.f, 0.f}, S[3] = {C.bg[0], C.bg[1], C.bg[2]}, Tc = 0.f, Tl = 1.f;
@@ -590,8 +590,8 @@ cudaError_t launch_translucent(const SceneView &S, const CamParams &C, const Opt
     cudaError_t e = launch_binning(S, C, Os, X, st, nullptr);
     if (e != cudaSuccess) return e;
     const int T = C.tiles_x * C.tiles_y;
-    k_tkeys<<<152 * 8, 256, 0, st>>>(X.s_list, X.s_off + T, X.s_tside, keys, X.status);
-    k_tsort<<<T, 256, 0, st>>>(X.s_off, keys, X.s_list, X.status);
+    k_tkeys<<<152 * 8, 256, 0, st>>>(X.s_list, X.s_tside, keys, X.status);
+    k_tsort<<<T, 256, 0, st>>>(X.s_rng, keys, X.s_list, X.status);
     if (front_first) k_traster<true><<<T, kRasterThreads, 0, st>>>(X, C, Os, w, out_rgb, out_T, out_front, out_last, out_Tlast, cover);
     else k_traster<false><<<T, kRasterThreads, 0, st>>>(X, C, Os, w, out_rgb, out_T, out_front, out_last, out_Tlast, cover);
     return cudaGetLastError();
@@ -610,8 +610,8 @@ cudaError_t launch_translucent_backward(const SceneView &S, const CamParams &C, 
     cudaError_t e = launch_binning(S, C, Os, X, st, nullptr);
     if (e != cudaSuccess) return e;
     const int T = C.tiles_x * C.tiles_y;
-    k_tkeys<<<152 * 8, 256, 0, st>>>(X.s_list, X.s_off + T, X.s_tside, keys, X.status);
-    k_tsort<<<T, 256, 0, st>>>(X.s_off, keys, X.s_list, X.status);
+    k_tkeys<<<152 * 8, 256, 0, st>>>(X.s_list, X.s_tside, keys, X.status);
+    k_tsort<<<T, 256, 0, st>>>(X.s_rng, keys, X.s_list, X.status);
     if ((e = cudaMemsetAsync(acc, 0, sizeof(long long) * kTAcc * (size_t)(S.N > 0 ? S.N : 1), st)) != cudaSuccess)
         return e;
     if ((e = launch_absmax(dL, 3 * (int64_t)C.W * C.H, gmax, st)) != cudaSuccess) return e;
