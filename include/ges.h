@@ -333,7 +333,7 @@ GES_API ges_status ges_render_batch(ges_scene *const *scenes, const ges_camera *
  * outputs are as in ges_render_ex (out_rgb required, the others may be
  * NULL); work is queued on `stream` and the call returns after that stream
  * has finished the render.  Intermediate data lives in one fixed device array
- * of 18 MiB that every GPU loading this library holds until the process
+ * of 26 MiB that every GPU loading this library holds until the process
  * exits.  Limits: n_surfels <= 65536, n_gaussians <= 65536, at most 16384
  * tiles of 16x16 pixels (e.g. 2048x2048), at most 1048576 tile entries per
  * primitive kind; larger inputs get GES_ERR_CAPACITY and a message.  The

@@ -80,11 +80,11 @@ struct ges_scene {
     DevBuf s_rec, s_rgb, g_rec, s_vis, g_vis;
     DevBuf s_cnt, g_cnt, s_rng, g_rng;
     DevBuf s_list, g_list;
-    DevBuf hist, base, vcount;     // local binning
+    DevBuf hist, base, vcount, order;   // local binning
     DevBuf status;                 // ST_WORDS per view slot
     DevBuf filt;                   // ges_compute_filter3d: cameras + one scratch word
     DevBuf g_aux;                  // Gaussian side data (2D Gaussians, geometry maps)
-    DevBuf t_side, t_keys;         // translucent render: surfel frames, sort keys
+    DevBuf t_side;                 // translucent render: surfel frames
     DevBuf t_acc;                  // backward passes: 64-bit fixed-point gradient sums + one word
     // ges_render_batch's batch graph (views of this and other scenes, with
     // this scene the first view's), kept while the calls keep the same key
@@ -240,12 +240,13 @@ ges_status ensure_scratch(ges_scene *s, int64_t T, int slots, cudaStream_t st)
         const LocalBins B = plan_local_bins(s->desc.n_surfels, s->desc.n_gaussians, sms);
         const int64_t P = std::max(B.Ps + B.Pg, 1), Tl = std::min<int64_t>(T, kLocalMaxTiles);
         const size_t row = (size_t)((Tl + 1) / 2) * 4;   // packed pairs of tiles
-        if ((e = s->hist.ensure(P * row)) || (e = s->base.ensure(2 * P * row)) || (e = s->vcount.ensure((size_t)P * 4)))
+        if ((e = s->hist.ensure(P * row)) || (e = s->base.ensure(2 * P * row)) || (e = s->vcount.ensure((size_t)P * 4)) ||
+            (e = s->order.ensure((size_t)Tl * kOrderItems * 4)))
             return cuda_fail(e, "scratch allocation (bins)");
     }
     if (s->s_cap == 0) s->s_cap = std::max<int64_t>((int64_t)1 << 20, 4 * s->desc.n_surfels);
     if (s->g_cap == 0) s->g_cap = std::max<int64_t>((int64_t)1 << 20, 4 * s->desc.n_gaussians);
-    if ((e = s->s_list.ensure(s->s_cap * 4)) || (e = s->g_list.ensure(s->g_cap * 4)))
+    if ((e = s->s_list.ensure(s->s_cap * 8)) || (e = s->g_list.ensure(s->g_cap * 8)))
         return cuda_fail(e, "scratch allocation (tile lists)");
     if (slots > s->status_slots) {
         if ((e = s->status.ensure((size_t)slots * ST_WORDS * 4))) return cuda_fail(e, "status allocation");
@@ -264,12 +265,13 @@ ViewScratch scratch_of(ges_scene *s, int slot)
     X.s_vis = (int *)s->s_vis.p; X.g_vis = (int *)s->g_vis.p;
     X.s_cnt = (int *)s->s_cnt.p; X.g_cnt = (int *)s->g_cnt.p;
     X.s_rng = (int2 *)s->s_rng.p; X.g_rng = (int2 *)s->g_rng.p;
-    X.s_list = (int *)s->s_list.p; X.g_list = (int *)s->g_list.p;
+    X.s_list = (uint2 *)s->s_list.p; X.g_list = (uint2 *)s->g_list.p;
     X.s_cap = s->s_cap; X.g_cap = s->g_cap;
     X.status = (unsigned *)s->status.p + (size_t)slot * ST_WORDS;
     X.hist = (unsigned *)s->hist.p;
     X.base = (unsigned *)s->base.p;
     X.vcount = (unsigned *)s->vcount.p;
+    X.order = (unsigned *)s->order.p;
     X.g_aux = (float4 *)s->g_aux.p;
     return X;
 }
@@ -433,8 +435,8 @@ ges_status ges_destroy_scene(ges_scene *s)
     if (!s) return GES_OK;
     cudaStreamSynchronize(s->stream);
     DevBuf *bufs[] = {&s->s_rec, &s->s_rgb, &s->g_rec, &s->s_vis, &s->g_vis, &s->s_cnt, &s->g_cnt, &s->s_rng,
-                      &s->g_rng, &s->s_list, &s->g_list, &s->hist, &s->base, &s->vcount,
-                       &s->status, &s->filt, &s->g_aux, &s->t_side, &s->t_keys, &s->t_acc};
+                      &s->g_rng, &s->s_list, &s->g_list, &s->hist, &s->base, &s->vcount, &s->order,
+                       &s->status, &s->filt, &s->g_aux, &s->t_side, &s->t_acc};
     for (DevBuf *b : bufs) b->release();
     if (s->bcache) batch_release(s->bcache);
     if (s->status_host) cudaFreeHost(s->status_host);
@@ -628,7 +630,7 @@ ges_status translucent_setup(ges_scene *s, const ges_camera *cam, const ges_rend
     const int64_t N = std::max<int64_t>(s->desc.n_surfels, 1);
     if ((r = ensure_scratch(s, (int64_t)C.tiles_x * C.tiles_y, 1, s->stream)) != GES_OK) return r;
     cudaError_t e;
-    if ((e = s->t_side.ensure((size_t)N * 64)) || (e = s->t_keys.ensure((size_t)s->s_cap * 8)))
+    if ((e = s->t_side.ensure((size_t)N * 64)))
         return cuda_fail(e, "scratch allocation (translucent)");
     X = scratch_of(s, 0);
     X.s_tside = (float4 *)s->t_side.p;
@@ -665,8 +667,8 @@ ges_status ges_render_translucent(ges_scene *s, const ges_camera *cam, const ges
         GES_CUDA(cudaMemsetAsync(X.status, 0, ST_WORDS * 4, s->stream));
         if (out_cover && s->desc.n_surfels > 0)
             GES_CUDA(cudaMemsetAsync(out_cover, 0, sizeof(int32_t) * (size_t)s->desc.n_surfels, s->stream));
-        cudaError_t e = launch_translucent(s->view, C, O, X, w, front_first != 0, (unsigned long long *)s->t_keys.p,
-                                           out_rgb, out_T, out_front, out_last, out_Tlast, out_cover, s->stream);
+        cudaError_t e = launch_translucent(s->view, C, O, X, w, front_first != 0, out_rgb,
+                                           out_T, out_front, out_last, out_Tlast, out_cover, s->stream);
         if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
         bool retry;
         if ((r = translucent_status(s, retry)) != GES_OK) return r;
@@ -694,7 +696,7 @@ ges_status ges_render_translucent_backward(ges_scene *s, const ges_camera *cam, 
         GES_CUDA(cudaMemsetAsync(X.status, 0, ST_WORDS * 4, s->stream));
         long long *acc = (long long *)s->t_acc.p;
         cudaError_t e = launch_translucent_backward(s->view, C, O, X, w, front_first != 0,
-                                                    (unsigned long long *)s->t_keys.p, dL_drgb, out_T, out_front,
+                                                    dL_drgb, out_T, out_front,
                                                     out_last, out_Tlast, acc, (unsigned *)(acc + (size_t)N * 18),
                                                     grads->s_pos, grads->s_rot, grads->s_scale, grads->s_w,
                                                     grads->s_sh, s->stream);
@@ -843,11 +845,12 @@ size_t batch_layout(ges_batch *b, const std::vector<SceneView> &S, const std::ve
         X.g_rng = (int2 *)take((size_t)T * 8);
         X.s_cap = b->s_cap[v];
         X.g_cap = b->g_cap[v];
-        X.s_list = (int *)take(b->s_cap[v] * 4);
-        X.g_list = (int *)take(b->g_cap[v] * 4);
+        X.s_list = (uint2 *)take(b->s_cap[v] * 8);
+        X.g_list = (uint2 *)take(b->g_cap[v] * 8);
         X.hist = (unsigned *)take((size_t)P * ((T + 1) / 2) * 4);
         X.base = (unsigned *)take((size_t)P * ((T + 1) / 2) * 8);
         X.vcount = (unsigned *)take((size_t)P * 4);
+        X.order = (unsigned *)take((size_t)T * 4);
         X.g_aux = S[v].gdim == 2 ? (float4 *)take(M * 32) : nullptr;
         X.g_col = (float4 *)take(M * 16);
         X.status = b->d_status + (size_t)v * ST_WORDS;
@@ -1124,10 +1127,8 @@ static ges_status batch_create(ges_scene *const *scenes, const ges_camera *cams,
         return cuda_fail(e, "cudaEventCreate");
     }
     auto drop_events = [&]() { cudaEventDestroy(e0); cudaEventDestroy(e1); };
-    // raster candidates: resident CTAs per SM (the 4-sample kernels are built
-    // for one CTA fewer)
-    const int d = O.samples == 4 ? 1 : 0;
-    const int kPerSm[] = {5 - d, 4 - d};
+    // raster candidates: CTAs per SM (all that are resident, or one fewer)
+    const int kPerSm[] = {kRasterCtas, kRasterCtas - 1};
     for (const auto &sh : shapes)
     for (int ri = 0; ri < nR; ++ri) {
         const std::vector<CamParams> Cs = shaped(sh);
@@ -1464,9 +1465,9 @@ constexpr size_t kNaSRng = kNaGCnt + kNaTileBytes;
 constexpr size_t kNaGRng = kNaSRng + 2 * kNaTileBytes;
 constexpr size_t kNaStatus = kNaGRng + 2 * kNaTileBytes;
 constexpr size_t kNaSList = na_align(kNaStatus + ST_WORDS * 4);
-constexpr size_t kNaGList = na_align(kNaSList + kNaMaxPairs * 4);
-constexpr size_t kNaBytes = na_align(kNaGList + kNaMaxPairs * 4);
-static_assert(kNaBytes <= (size_t)18 << 20, "fixed scratch exceeds its stated 18 MiB");
+constexpr size_t kNaGList = na_align(kNaSList + kNaMaxPairs * 8);
+constexpr size_t kNaBytes = na_align(kNaGList + kNaMaxPairs * 8);
+static_assert(kNaBytes <= (size_t)26 << 20, "fixed scratch exceeds its stated 26 MiB");
 
 constexpr int kNaMaxDevices = 64;
 std::once_flag g_na_once[kNaMaxDevices];
@@ -1525,7 +1526,7 @@ extern "C" GES_API ges_status ges_render_noalloc(const ges_scene_desc *desc, con
     X.s_vis = (int *)(base + kNaSVis); X.g_vis = (int *)(base + kNaGVis);
     X.s_cnt = (int *)(base + kNaSCnt); X.g_cnt = (int *)(base + kNaGCnt);
     X.s_rng = (int2 *)(base + kNaSRng); X.g_rng = (int2 *)(base + kNaGRng);
-    X.s_list = (int *)(base + kNaSList); X.g_list = (int *)(base + kNaGList);
+    X.s_list = (uint2 *)(base + kNaSList); X.g_list = (uint2 *)(base + kNaGList);
     X.s_cap = kNaMaxPairs; X.g_cap = kNaMaxPairs;
     X.status = (unsigned *)(base + kNaStatus);
     // the array keeps the previous call's contents: clear the tile counters

@@ -17,10 +17,12 @@ namespace ges {
 
 constexpr int kTile = 16;               // default binning tile edge (pixels): 16x16
 constexpr int kTileShift = 4;           // log2 kTile
-constexpr int kRasterThreads = 256;     // 8 warps, each an 8x4 pixel block
+constexpr int kRasterThreads = 256;     // 8 warps
+constexpr int kRasterCtas = 4;          // resident raster CTAs per SM (64 registers per thread)
 constexpr int kWarpW = 8, kWarpH = 4;
-// A binning tile holds the 8 warps' blocks: 2^tsx x 2^tsy pixels with
-// tsx + tsy = 8 and tsx in [3, 6] (8x32, 16x16, 32x8, 64x4).
+// A binning tile is 2^tsx x 2^tsy pixels, tsx >= 3 and tsy >= 2: whole 8x4
+// blocks, at most kMaskBits block columns and rows together.
+constexpr int kMaskBits = 12;
 
 // status word layout (uint32 words)
 enum : int {
@@ -31,10 +33,11 @@ enum : int {
     ST_GPAIRS = 4,        // Gaussian tile pairs
     ST_SFRAG = 5,         // surfel fragments inside their discs (work count)
     ST_GFRAG = 6,         // Gaussian pixel terms with alpha >= alpha_min (work count)
-    ST_RETIRED = 7,       // batch raster: tiles of this view finished
-    ST_TDONE = 8,         // batch raster: %globaltimer (ns, 64-bit, words 8-9) when the last tile finished
+    ST_RETIRED = 7,       // batch raster: blocks of this view finished
+    ST_TDONE = 8,         // batch raster: %globaltimer (ns, 64-bit, words 8-9) when the last one finished
     ST_SCUR = 10,         // tile-list space handed out, surfels (64-bit, words 10-11)
     ST_GCUR = 12,         // the same for the Gaussians (words 12-13)
+    ST_ITEMS = 14,        // one view: items in the order array; batch: its tiles shared by a CTA's warps
     ST_WORDS = 16,
 };
 enum : unsigned { FLAG_SOVF = 1u, FLAG_GOVF = 2u, FLAG_BADQ = 4u };
@@ -76,12 +79,12 @@ struct ViewScratch {
     float4 *s_rgb;        // [N]     surfel colours
     float4 *g_rec;        // [M][4]  Gaussian raster records
     // visible primitives: with local bins, per-CTA segments of 16-byte entries
-    // (id, bbox lo, bbox hi, -), 16 B per primitive; with atomic binning one
-    // id per entry
+    // (id, bbox lo, bbox hi, cull key), 16 B per primitive; with atomic binning
+    // one id per entry
     int *s_vis, *g_vis;
     int *s_cnt, *g_cnt;   // [T]     per-tile counts (atomic binning; zero between renders)
     int2 *s_rng, *g_rng;  // [T]     (start, end) of each tile's list
-    int *s_list, *g_list; // tile lists
+    uint2 *s_list, *g_list; // tile lists: (id, cull word), see list_word
     int64_t s_cap, g_cap; // list capacities (entries)
     unsigned *status;     // [ST_WORDS]
     // local binning (per-CTA primitive ranges with shared-memory histograms);
@@ -89,6 +92,10 @@ struct ViewScratch {
     unsigned *hist = nullptr;    // [P][ceil(T/2)] packed 16-bit per-CTA tile counts
     unsigned *base = nullptr;    // [P][2 ceil(T/2)] per-CTA start inside each tile's list
     unsigned *vcount = nullptr;  // [P] visible primitives per CTA
+    // raster items, the costliest first (written by the fill; see order_body);
+    // one view: up to kOrderItems per tile, a batch: one per tile; null: the
+    // tiles as they lie
+    unsigned *order = nullptr;
     // [M][2] side data of each Gaussian, written when the render needs it:
     // 2D Gaussians (rgb, log2 sigma'), (normal, log2(alpha_min / sigma'));
     // 3D Gaussians with geometry outputs (normal, centre depth), unused
@@ -106,6 +113,8 @@ struct LocalBins {
     int Ps, Pg;           // CTAs over surfels, over Gaussians
     int64_t Rs, Rg;       // primitives per CTA
 };
+constexpr int kOrderItems = 8;          // blocks of a binning tile
+constexpr int kShareSlots = 152 * kRasterCtas;   // resident raster CTAs of the GPU
 constexpr int kLocalMaxTiles = 32768;   // shared-memory cursors of the fill: 4 B per tile
 
 // One view of a batch (device table entry).  The batch kernels find their view
@@ -149,7 +158,7 @@ cudaError_t launch_batch(const BatchView *d_views, const BatchPlan &P, const Opt
                          cudaStream_t st, cudaEvent_t *ev, bool ids);
 LocalBins plan_local_bins_per_cta(int64_t N, int64_t M, int64_t prims_per_cta);
 constexpr int kPrepThreads = 512;
-constexpr int kFillThreads = 1024;
+constexpr int kFillThreads = 768;       // two CTAs per SM: 42 registers each (1024 threads spill, and take 8 % longer)
 constexpr int kAllocTiles = 1024;       // tiles per CTA of the list allocation (atomic binning)
 constexpr int kColTiles = 64;           // tiles per CTA of the column scan
 LocalBins plan_local_bins(int64_t N, int64_t M, int num_sms);
@@ -166,16 +175,16 @@ cudaError_t launch_binning(const SceneView &S, const CamParams &C, const OptPara
                            cudaStream_t st, cudaEvent_t *ev);
 
 // Translucent-surfel render (Sec. 4.1) of one view: binning of the surfels
-// (X.s_tside must be set), per-tile sort, blend.  keys: one 64-bit word per
-// tile-list entry.  cover (or null): per-surfel counts of frontmost pixels, added.
+// (X.s_tside must be set; the lists then hold sort keys), per-tile sort, blend.
+// cover (or null): per-surfel counts of frontmost pixels, added.
 cudaError_t launch_translucent(const SceneView &S, const CamParams &C, const OptParams &O, const ViewScratch &X,
-                               const float *w, bool front_first, unsigned long long *keys, float *out_rgb,
+                               const float *w, bool front_first, float *out_rgb,
                                float *out_T, int32_t *out_front, int32_t *out_last, float *out_Tlast, int32_t *cover,
                                cudaStream_t st);
 // Its backward: acc [N][18] 64-bit words and gmax (one word) are scratch.
 cudaError_t launch_translucent_backward(const SceneView &S, const CamParams &C, const OptParams &O,
                                         const ViewScratch &X, const float *w, bool front_first,
-                                        unsigned long long *keys, const float *dL, const float *in_T,
+                                        const float *dL, const float *in_T,
                                         const int32_t *in_front, const int32_t *in_last, const float *in_Tlast,
                                         long long *acc, unsigned *gmax, float *g_pos, float *g_rot, float *g_scale,
                                         float *g_w, float *g_sh, cudaStream_t st);
@@ -480,6 +489,44 @@ __device__ __forceinline__ bool quat_to_rot(float w, float x, float y, float z, 
     R[3] = 2.f * (x * y + w * z); R[4] = 1.f - 2.f * (x * x + z * z); R[5] = 2.f * (y * z - w * x);
     R[6] = 2.f * (x * z - w * y); R[7] = 2.f * (y * z + w * x); R[8] = 1.f - 2.f * (x * x + y * y);
     return true;
+}
+
+// The cull word of a tile-list entry: the low nb = block columns + block rows
+// bits say which columns (low) and rows of the tile's 8x4 blocks the
+// primitive's bbox touches, the bits above are its cull key's, a float rounded
+// so that the whole word, read as a float, is still on the safe side: not
+// below a surfel's largest 1/z, not above a Gaussian's d - eps.  A key beyond
+// the finite floats becomes a NaN, which the negated compares keep.
+__device__ __forceinline__ unsigned surfel_key_bits(float izmax, int nb)
+{
+    const unsigned m = (1u << nb) - 1u;
+    return (__float_as_uint(izmax) + m) & ~m;          // izmax > 0: away from zero
+}
+__device__ __forceinline__ unsigned gauss_key_bits(float key, int nb)
+{
+    const unsigned m = (1u << nb) - 1u, b = __float_as_uint(key);
+    if (b & 0x80000000u) return (b + m) & ~m;          // away from zero, the mask bits too
+    return b > 2u * m + 1u ? (b & ~m) - (m + 1u) : 0x80000000u;
+}
+// nb of a tile shape
+__device__ __forceinline__ int mask_bits(int tsx, int tsy) { return (1 << (tsx - 3)) + (1 << (tsy - 2)); }
+// block columns of the tiles in column tx, block rows of those in row ty, that
+// pixels x0..x1, y0..y1 touch (they touch the tile)
+__device__ __forceinline__ unsigned col_mask(int x0, int x1, int tx, int tsx)
+{
+    const int c0 = max(x0 - (tx << tsx), 0) >> 3, c1 = min(x1 - (tx << tsx), (1 << tsx) - 1) >> 3;
+    return (2u << c1) - (1u << c0);
+}
+__device__ __forceinline__ unsigned row_mask(int y0, int y1, int ty, int tsx, int tsy)
+{
+    const int r0 = max(y0 - (ty << tsy), 0) >> 2, r1 = min(y1 - (ty << tsy), (1 << tsy) - 1) >> 2;
+    return ((2u << r1) - (1u << r0)) << (1 << (tsx - 3));
+}
+// order-preserving float -> uint
+__device__ __forceinline__ unsigned depth_key(float z)
+{
+    const unsigned b = __float_as_uint(z);
+    return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
 }
 
 __device__ __forceinline__ unsigned pack_xy(int x, int y) { return (unsigned)x | ((unsigned)y << 16); }

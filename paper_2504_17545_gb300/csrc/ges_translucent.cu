@@ -8,8 +8,8 @@
 // by r = sqrt(surfel_r2): rho = r^2 (A^2 + B^2)/iz^2).
 //
 //   binning      the opaque preprocess (surfels only), which also writes each
-//                surfel's camera-space frame for the backward;
-//   k_tkeys      per tile-list entry the key (centre camera depth, index);
+//                surfel's camera-space frame for the backward and fills the
+//                lists with the keys (centre camera depth, index);
 //   k_tsort      per tile, the list sorted by that key (bitonic, in shared
 //                memory up to 4096 entries, in global memory beyond);
 //   k_traster    per pixel: the frontmost contributor (least depth at the
@@ -36,25 +36,6 @@ constexpr int kTAcc = 18;               // gradient terms accumulated per surfel
 
 __device__ __forceinline__ unsigned lane_idx() { return threadIdx.x & 31u; }
 
-// order-preserving float -> uint
-__device__ __forceinline__ unsigned depth_key(float z)
-{
-    const unsigned b = __float_as_uint(z);
-    return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-}
-
-__global__ void __launch_bounds__(256) k_tkeys(const int *__restrict__ list,
-                                               const float4 *__restrict__ tside, unsigned long long *keys,
-                                               const unsigned *status)
-{
-    if (status[ST_FLAGS] & FLAG_SOVF) return;     // lists not filled; the count exceeds the capacity
-    const int n = (int)status[ST_SPAIRS];
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int id = list[i];
-        keys[i] = ((unsigned long long)depth_key(tside[4 * (int64_t)id].z) << 32) | (unsigned)id;
-    }
-}
-
 // Ascending bitonic sort of a[0..n) (m = the next power of two); pairs whose
 // upper index is >= n are skipped, which equals padding with +infinity
 // because every compare-exchange moves the smaller key to the lower index.
@@ -79,23 +60,24 @@ __device__ __forceinline__ void bitonic(unsigned long long *a, int n, int m)
     }
 }
 
-__global__ void __launch_bounds__(256) k_tsort(const int2 *__restrict__ rng, unsigned long long *keys, int *list,
-                                               const unsigned *status)
+// The list entries are the sort keys: (id, depth key) read as one 64-bit word
+// with the depth key above.
+__global__ void __launch_bounds__(256) k_tsort(const int2 *__restrict__ rng, uint2 *list, const unsigned *status)
 {
     __shared__ unsigned long long sk[kSortCap];
     if (status[ST_FLAGS] & FLAG_SOVF) return;
     const int a = rng[blockIdx.x].x, n = rng[blockIdx.x].y - a;
     if (n <= 1) return;
+    unsigned long long *keys = reinterpret_cast<unsigned long long *>(list) + a;
     int m = 1;
     while (m < n) m <<= 1;
     if (n <= kSortCap) {
-        for (int k = threadIdx.x; k < n; k += blockDim.x) sk[k] = keys[a + k];
+        for (int k = threadIdx.x; k < n; k += blockDim.x) sk[k] = keys[k];
         __syncthreads();
         bitonic(sk, n, m);
-        for (int k = threadIdx.x; k < n; k += blockDim.x) list[a + k] = (int)(unsigned)(sk[k] & 0xffffffffull);
+        for (int k = threadIdx.x; k < n; k += blockDim.x) keys[k] = sk[k];
     } else {
-        bitonic(keys + a, n, m);
-        for (int k = threadIdx.x; k < n; k += blockDim.x) list[a + k] = (int)(unsigned)(keys[a + k] & 0xffffffffull);
+        bitonic(keys, n, m);
     }
 }
 
@@ -162,7 +144,7 @@ __global__ void __launch_bounds__(kRasterThreads, 4)
     const int t = threadIdx.x;
     auto stage = [&](int base) {
         if (base + t < s1) {
-            const int id = X.s_list[base + t];
+            const int id = (int)X.s_list[base + t].x;
             const float4 *rp = X.s_rec + 4 * (int64_t)id;
             ss[0][t] = rp[0]; ss[1][t] = rp[1]; ss[2][t] = rp[2];
             const float4 r3 = rp[3];
@@ -358,7 +340,7 @@ __global__ void __launch_bounds__(kRasterThreads, 3)
     for (int cbase = ((nl - 1) / kRasterThreads) * kRasterThreads; nl > 0 && cbase >= 0; cbase -= kRasterThreads) {
         __syncthreads();
         if (s0 + cbase + t < s1 && cbase + t < nl) {
-            const int id = X.s_list[s0 + cbase + t];
+            const int id = (int)X.s_list[s0 + cbase + t].x;
             const float4 *rp = X.s_rec + 4 * (int64_t)id;
             ss[0][t] = rp[0]; ss[1][t] = rp[1]; ss[2][t] = rp[2];
             const float4 r3 = rp[3];
@@ -581,7 +563,7 @@ __global__ void __launch_bounds__(256) k_contrib(SceneView S, CamParams C, OptPa
 }  // namespace
 
 cudaError_t launch_translucent(const SceneView &S, const CamParams &C, const OptParams &O, const ViewScratch &X,
-                               const float *w, bool front_first, unsigned long long *keys, float *out_rgb,
+                               const float *w, bool front_first, float *out_rgb,
                                float *out_T, int32_t *out_front, int32_t *out_last, float *out_Tlast, int32_t *cover,
                                cudaStream_t st)
 {
@@ -590,8 +572,7 @@ cudaError_t launch_translucent(const SceneView &S, const CamParams &C, const Opt
     cudaError_t e = launch_binning(S, C, Os, X, st, nullptr);
     if (e != cudaSuccess) return e;
     const int T = C.tiles_x * C.tiles_y;
-    k_tkeys<<<152 * 8, 256, 0, st>>>(X.s_list, X.s_tside, keys, X.status);
-    k_tsort<<<T, 256, 0, st>>>(X.s_rng, keys, X.s_list, X.status);
+    k_tsort<<<T, 256, 0, st>>>(X.s_rng, X.s_list, X.status);
     if (front_first) k_traster<true><<<T, kRasterThreads, 0, st>>>(X, C, Os, w, out_rgb, out_T, out_front, out_last, out_Tlast, cover);
     else k_traster<false><<<T, kRasterThreads, 0, st>>>(X, C, Os, w, out_rgb, out_T, out_front, out_last, out_Tlast, cover);
     return cudaGetLastError();
@@ -599,7 +580,7 @@ cudaError_t launch_translucent(const SceneView &S, const CamParams &C, const Opt
 
 cudaError_t launch_translucent_backward(const SceneView &S, const CamParams &C, const OptParams &O,
                                         const ViewScratch &X, const float *w, bool front_first,
-                                        unsigned long long *keys, const float *dL, const float *in_T,
+                                        const float *dL, const float *in_T,
                                         const int32_t *in_front, const int32_t *in_last, const float *in_Tlast,
                                         long long *acc, unsigned *gmax, float *g_pos, float *g_rot, float *g_scale,
                                         float *g_w, float *g_sh, cudaStream_t st)
@@ -610,8 +591,7 @@ cudaError_t launch_translucent_backward(const SceneView &S, const CamParams &C, 
     cudaError_t e = launch_binning(S, C, Os, X, st, nullptr);
     if (e != cudaSuccess) return e;
     const int T = C.tiles_x * C.tiles_y;
-    k_tkeys<<<152 * 8, 256, 0, st>>>(X.s_list, X.s_tside, keys, X.status);
-    k_tsort<<<T, 256, 0, st>>>(X.s_rng, keys, X.s_list, X.status);
+    k_tsort<<<T, 256, 0, st>>>(X.s_rng, X.s_list, X.status);
     if ((e = cudaMemsetAsync(acc, 0, sizeof(long long) * kTAcc * (size_t)(S.N > 0 ? S.N : 1), st)) != cudaSuccess)
         return e;
     if ((e = launch_absmax(dL, 3 * (int64_t)C.W * C.H, gmax, st)) != cudaSuccess) return e;
