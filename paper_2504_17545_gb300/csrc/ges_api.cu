@@ -1148,6 +1148,12 @@ static ges_status batch_create(ges_scene *const *scenes, const ges_camera *cams,
                 P.total_colscan += (b->views[v].T + kColTiles - 1) / kColTiles;
                 P.max_T = std::max(P.max_T, b->views[v].T);
             }
+            // one set-up kernel for all views: staged rows only if every view's are
+            P.stage_bytes = staged_row_bytes(S[0], P.max_T);
+            for (int v = 1; v < n_views; ++v) {
+                const int row = staged_row_bytes(S[v], P.max_T);
+                P.stage_bytes = row && P.stage_bytes ? std::max(P.stage_bytes, row) : 0;
+            }
             std::memcpy(b->h_table, b->views.data(), sizeof(BatchView) * n_views);
             if ((e = upload_prep_map(b, P)) != cudaSuccess) {
                 drop_events();

@@ -97,13 +97,17 @@ __device__ __forceinline__ GaussRec gauss_rec3(float4 a, float4 b, float4 c)
     return g;
 }
 
+// Where a set-up's colours (Eq. 1) come from.
+enum ColourFrom : int {
+    COL_PASS = 0,     // the batch's colour pass (ran before for the Gaussians, surfels need nothing)
+    COL_HERE = 1,     // evaluated with the geometry, the SH row read by its thread
+    COL_STAGED = 2,   // evaluated later from an SH row staged in shared memory (see sh_stage)
+};
 // Set up primitive i of the given kind; on success write its record and
-// return its pixel bbox.
+// return its pixel bbox and cull key.
 // kGd: the scene's Gaussian kind (a template argument, so that each kernel
-// carries only its own set-up code)
-// kCol false: leave the colour (Eq. 1) to the batch's colour pass; only the
-// geometry is set up and stored here.
-template <int kGd, bool kTr = false, bool kCol = true>
+// carries only its own set-up code).  kCol: ColourFrom.
+template <int kGd, bool kTr = false, int kCol = COL_HERE>
 __device__ __forceinline__ bool setup_and_store(const SceneView &S, const CamParams &C, const OptParams &O,
                                                 const ViewScratch &X, bool surf, int64_t i, int &x0, int &y0,
                                                 int &x1, int &y1, unsigned &key)
@@ -117,7 +121,7 @@ __device__ __forceinline__ bool setup_and_store(const SceneView &S, const CamPar
         if (!o.valid_quat) atomicOr(X.status + ST_FLAGS, FLAG_BADQ);
         if (!o.visible) return false;
         store_rec(X.s_rec + 4 * i, o.rec);
-        if (kCol) {
+        if (kCol == COL_HERE) {
             surfel_colour(S, i, o);
             X.s_rgb[i] = make_float4(o.rgb[0], o.rgb[1], o.rgb[2], 0.f);
         }
@@ -126,7 +130,7 @@ __device__ __forceinline__ bool setup_and_store(const SceneView &S, const CamPar
         key = kTr ? depth_key(X.s_tside[4 * i].z) : surfel_key_bits(o.rec.izmax, nb);
     } else {
         GaussOut o;
-        if (kGd == 2) gauss2d_setup(S, C, O, i, o, kCol);
+        if (kGd == 2) gauss2d_setup(S, C, O, i, o, kCol == COL_HERE);
         else gauss_geom(S, C, O, i, o);
         if (!o.valid_quat) atomicOr(X.status + ST_FLAGS, FLAG_BADQ);
         if (!o.visible) return false;
@@ -139,21 +143,23 @@ __device__ __forceinline__ bool setup_and_store(const SceneView &S, const CamPar
             dst[1] = make_float4(o.rec.la, o.rec.lb, o.rec.lc, o.rec.sigma);
             dst[3] = make_float4(__int_as_float(o.rec.id), __uint_as_float(o.rec.bb_lo),
                                  __uint_as_float(o.rec.bb_hi), o.rec.pad);
-            if (kCol) {
+            if (kCol == COL_HERE) {
                 gauss_colour(S, i, o);
                 dst[2] = make_float4(o.rec.key, colour_q(o.rec.r), colour_q(o.rec.g), colour_q(o.rec.b));
-            } else {
+            } else if (kCol == COL_PASS) {
                 const float4 c = X.g_col[i];   // the colour pass's colour
                 dst[2] = make_float4(o.rec.key, c.x, c.y, c.z);
+            } else {
+                dst[2].x = o.rec.key;          // the staged colour joins it
             }
         }
         if (kGd == 2 || O.geo) {
             float4 a0 = o.aux[0];
-            if (kGd == 2 && !kCol) {
+            if (kGd == 2 && kCol == COL_PASS) {
                 const float4 c = X.g_col[i];   // the colour pass's colour
                 a0.x = c.x; a0.y = c.y; a0.z = c.z;
             }
-            X.g_aux[2 * i] = a0;
+            X.g_aux[2 * i] = a0;               // (2D: a staged colour joins log2 sigma')
             X.g_aux[2 * i + 1] = o.aux[1];
         }
         x0 = o.x0; y0 = o.y0; x1 = o.x1; y1 = o.y1;
@@ -161,6 +167,74 @@ __device__ __forceinline__ bool setup_and_store(const SceneView &S, const CamPar
         key = gauss_key_bits(kGd == 2 ? 1.f / o.drec.izmax - o.drec.pad : o.rec.key, nb);
     }
     return true;
+}
+
+// Staged SH rows (16 coefficients per channel: 192 bytes in FP32, 96 in 16
+// bits).  A warp copies the rows of its visible primitives to its own shared
+// space, 16 bytes per lane and consecutive lanes consecutive bytes, while it
+// sets up the next 32 primitives, and evaluates the colours afterwards.  A row
+// per thread read directly (12 loads of 16 bytes, 192 bytes apart between the
+// lanes: 32 cache lines per load) added its whole time to the set-up's: of the
+// preprocess of a 1080p view (1M + 300k, FP32) 110 us, 47 were the colours;
+// staged it takes 90 (200k + 2.5M: 195 -> 163; 2.25M + 750k in FP16: 217 -> 186).
+// The copies must cost few instructions: with the chunk's place worked out one
+// by one the set-up issued 84M instead of 56M instructions and gained nothing.
+// kChunks 16-byte chunks per row, 12 or 6.  Chunk c of row r lies at c ^ swz(r),
+// which spreads equal chunks of eight consecutive rows over all banks.
+constexpr int kShRows = 16;     // basis functions of a staged row
+template <int kChunks>
+__device__ __forceinline__ int sh_swz(int r) { return kChunks == 12 ? r >> 1 & 3 : r >> 2 & 1; }
+
+template <int kChunks>
+__device__ __forceinline__ void sh_stage(const void *sh, int64_t i0, unsigned vis, unsigned char *st)
+{
+    // the lane's chunks: number 32 j + lane of the 32 rows; three of them
+    // (j = 0, 1, 2) end on a whole number of rows, then the pattern repeats
+    constexpr int kRep = kChunks / 3, kRepRows = 96 / kChunks;
+    const unsigned base = (unsigned)__cvta_generic_to_shared(st);
+    const int lane = (int)lane_id();
+    const unsigned char *src = reinterpret_cast<const unsigned char *>(sh) + (i0 * kChunks + lane) * 16;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const int g = 32 * j + lane, r = kChunks == 12 ? (g * 43) >> 9 : (g * 43) >> 8, c = g - kChunks * r;
+        const unsigned dst = base + (unsigned)(16 * (kChunks * r + (c ^ sh_swz<kChunks>(r)))), v = vis >> r;
+#pragma unroll
+        for (int m = 0; m < kRep; ++m)
+            if (v & (1u << (kRepRows * m)))
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
+                             :: "r"(dst + 16u * kChunks * kRepRows * m), "l"(src + 512 * j + 1536 * m) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// The colour from the lane's staged row, by sh_colour's operations in their order.
+template <int kChunks>
+__device__ __forceinline__ void sh_staged_colour(const unsigned char *st, bool half, const float *dir, float *rgb)
+{
+    const int lane = (int)lane_id();
+    float Y[kShRows];
+    sh_basis(kShRows, dir[0], dir[1], dir[2], Y);
+    float v[3] = {0.5f, 0.5f, 0.5f};
+    const uint4 *row = reinterpret_cast<const uint4 *>(st) + kChunks * lane;
+    const int k0 = sh_swz<kChunks>(lane);
+#pragma unroll
+    for (int q = 0; q < kChunks; ++q) {
+        const uint4 x = row[q ^ k0];
+        const unsigned e[4] = {x.x, x.y, x.z, x.w};
+        constexpr int kN = kChunks == 12 ? 4 : 8;
+#pragma unroll
+        for (int k = 0; k < kN; ++k) {
+            float c;
+            if (kChunks == 12) {
+                c = __uint_as_float(e[k]);
+            } else {
+                const unsigned short h = (unsigned short)(k & 1 ? e[k / 2] >> 16 : e[k / 2] & 0xffffu);
+                c = half ? __half2float(__ushort_as_half(h)) : __bfloat162float(__ushort_as_bfloat16(h));
+            }
+            v[(kN * q + k) % 3] = fmaf(c, Y[(kN * q + k) / 3], v[(kN * q + k) % 3]);
+        }
+    }
+    rgb[0] = fmaxf(v[0], 0.f); rgb[1] = fmaxf(v[1], 0.f); rgb[2] = fmaxf(v[2], 0.f);
 }
 
 // ---------------------------------------------------------------------------
@@ -201,15 +275,42 @@ __device__ __forceinline__ void for_tiles(bool on, const int4 &c, int tsx, int t
 
 // CTA c of a view: its range of primitives.  hist: ceil(T/2) shared words
 // (two 16-bit counters each); vcnt: a shared counter.
-// kKind: 0 both kinds (CTA c < B.Ps: surfels), 1 surfel ranges only, 2
-// Gaussian ranges only (a launch per kind gives each its own registers)
-template <int kGd, bool kTr = false, int kKind = 0, bool kCol = true>
+// kKind: 1 a surfel range, 2 a Gaussian range (each its own code)
+// kCol COL_STAGED: the shared memory after the histogram holds an SH row per
+// thread.
+template <int kGd, bool kTr, int kKind, int kCol>
 __device__ __forceinline__ void prep_local_body(const SceneView &S, const CamParams &C, const OptParams &O,
                                                 const ViewScratch &X, const LocalBins &B, int c, unsigned *hist,
                                                 unsigned &vcnt)
 {
     const int T = C.tiles_x * C.tiles_y, words = (T + 1) >> 1;
-    const bool surf = kKind == 1 ? true : (kKind == 2 ? false : c < B.Ps);
+    const int row_bytes = 3 * kShRows * (S.sh_dtype == GES_F32 ? 4 : 2);
+    unsigned char *stage = reinterpret_cast<unsigned char *>(hist + ((words + 3) & ~3)) +
+                           (size_t)(threadIdx.x >> 5) * 32 * row_bytes;
+    constexpr bool surf = kKind == 1;
+    unsigned pending = 0;   // the lanes whose rows are being staged
+    // The colours of round i's staged rows.  Nothing but the mask is carried
+    // over from the set-up: the position and the word beside the colour are
+    // read again (from L2), which is cheaper than spilling them.
+    const auto colour = [&](int64_t i) {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncwarp();
+        if (pending >> lane_id() & 1u) {
+            const float *pos = surf ? S.s_pos : S.g_pos;
+            float dir[3], L, rgb[3];
+            view_dir(C, __ldg(pos + 3 * i), __ldg(pos + 3 * i + 1), __ldg(pos + 3 * i + 2), dir, L);
+            if (S.sh_dtype == GES_F32) sh_staged_colour<12>(stage, false, dir, rgb);
+            else sh_staged_colour<6>(stage, S.sh_dtype == GES_F16, dir, rgb);
+            if (surf) {
+                X.s_rgb[i] = make_float4(rgb[0], rgb[1], rgb[2], 0.f);
+            } else {
+                const float r = colour_q(rgb[0]), g = colour_q(rgb[1]), b = colour_q(rgb[2]);
+                if (kGd == 2) X.g_aux[2 * i] = make_float4(r, g, b, X.g_aux[2 * i].w);
+                else X.g_rec[4 * i + 2] = make_float4(X.g_rec[4 * i + 2].x, r, g, b);
+            }
+        }
+        __syncwarp();       // the rows are read: the space is free
+    };
     const int64_t R = surf ? B.Rs : B.Rg, n = surf ? S.N : S.M;
     const int64_t beg = (int64_t)(surf ? c : c - B.Ps) * R;
     const int64_t end = beg + R < n ? beg + R : n;
@@ -227,6 +328,14 @@ __device__ __forceinline__ void prep_local_body(const SceneView &S, const CamPar
         const bool vis = i < end && setup_and_store<kGd, kTr, kCol>(S, C, O, X, surf, i, x0, y0, x1, y1, key);
         const int4 entry = make_int4((int)i, (int)pack_xy(x0, y0), (int)pack_xy(x1, y1), (int)key);
         const unsigned m = __ballot_sync(0xffffffffu, vis);
+        if (kCol == COL_STAGED) {
+            // the rows asked for a round ago are here: their colours, then this round's rows
+            if (i0 != beg) colour(i - kPrepThreads);
+            pending = m;
+            const void *sh = surf ? S.s_sh : S.g_sh;
+            if (S.sh_dtype == GES_F32) sh_stage<12>(sh, i - (int64_t)lane_id(), m, stage);
+            else sh_stage<6>(sh, i - (int64_t)lane_id(), m, stage);
+        }
         if (m) {
             const int leader = __ffs(m) - 1;
             unsigned b = 0;
@@ -239,6 +348,8 @@ __device__ __forceinline__ void prep_local_body(const SceneView &S, const CamPar
             atomicAdd(hist + (t >> 1), (t & 1) ? 65536u : 1u);
         });
     }
+    if (kCol == COL_STAGED && beg < end)
+        colour(beg + (end - beg - 1) / kPrepThreads * kPrepThreads + threadIdx.x);
     __syncthreads();
     unsigned *row = X.hist + (size_t)c * words;
     for (int w = threadIdx.x; w < words; w += kPrepThreads) row[w] = hist[w];
@@ -248,13 +359,15 @@ __device__ __forceinline__ void prep_local_body(const SceneView &S, const CamPar
     }
 }
 
-template <int kGd, bool kTr = false>
+template <int kGd, bool kTr, int kCol>
 __global__ void __launch_bounds__(kPrepThreads, 2) k_prep_local(SceneView S, CamParams C, OptParams O,
                                                                 ViewScratch X, LocalBins B)
 {
-    extern __shared__ unsigned hist[];
+    extern __shared__ __align__(16) unsigned hist[];
     __shared__ unsigned vcnt;
-    prep_local_body<kGd, kTr>(S, C, O, X, B, blockIdx.x, hist, vcnt);
+    // the two kinds' code apart, so that neither's registers count for the other
+    if ((int)blockIdx.x < B.Ps) prep_local_body<kGd, kTr, 1, kCol>(S, C, O, X, B, blockIdx.x, hist, vcnt);
+    else prep_local_body<kGd, kTr, 2, kCol>(S, C, O, X, B, blockIdx.x, hist, vcnt);
 }
 
 // Space for the lists of the tiles whose totals a warp holds (n tiles on each
@@ -1090,14 +1203,13 @@ __global__ void __launch_bounds__(kRasterThreads, kRasterCtas)
              int32_t *__restrict__ out_id, float *__restrict__ aux, GeoMaps geo)
 {
     __shared__ WarpSpace<kS, kG, kGeo> space[kRasterWarps];
-    if (X.status[ST_FLAGS] & (FLAG_SOVF | FLAG_GOVF)) return;
     // one CTA per item (persistent CTAs that take items from a counter took 10 %
-    // longer: two barriers per item); the grid has room for the most there can be
+    // longer: two barriers per item); the grid has room for the most there can be,
+    // and the order array for the grid, so that its word is read with the status
     unsigned item = blockIdx.x;
-    if (X.order) {
-        if (item >= X.status[ST_ITEMS]) return;
-        item = X.order[item];
-    }
+    if (X.order) item = X.order[blockIdx.x];
+    if (X.status[ST_FLAGS] & (FLAG_SOVF | FLAG_GOVF)) return;
+    if (X.order && blockIdx.x >= X.status[ST_ITEMS]) return;
     const int tile = (int)(item & 0xffffffu), nb = 1 << (C.tsx + C.tsy - 5);
     if (item >> 24) {
         raster_block<kS, kG, kGeo, true>(X, C, O, out_rgb, out_depth, out_id, aux, geo, tile, (int)(item >> 24) - 1,
@@ -1137,11 +1249,11 @@ __device__ __forceinline__ void load_view(const BatchView *V, int v, BatchView &
 // kernel per kind keeps the one from spilling for the other.  kCol: the
 // colours too (a batch whose scenes each have one view; otherwise the colour
 // pass evaluates them for all views of a scene at once).
-template <int kGd, int kKind, bool kCol>
+template <int kGd, int kKind, int kCol>
 __global__ void __launch_bounds__(kPrepThreads, 2) k_bprep(const BatchView *V, const int2 *__restrict__ map,
                                                           OptParams O, unsigned long long *t0)
 {
-    extern __shared__ unsigned hist[];
+    extern __shared__ __align__(16) unsigned hist[];
     __shared__ unsigned vcnt;
     __shared__ __align__(16) unsigned char bv_raw[sizeof(BatchView)];
     BatchView &bv = *reinterpret_cast<BatchView *>(bv_raw);
@@ -1341,6 +1453,8 @@ __global__ void __launch_bounds__(kRasterThreads, kRasterCtas) k_braster(const B
 
 }  // namespace
 
+static size_t stage_smem(int T, int row_bytes);
+
 cudaError_t launch_batch(const BatchView *d_views, const BatchPlan &P, const OptParams &O, unsigned *work_counter,
                          cudaStream_t st, cudaEvent_t *ev, bool ids)
 {
@@ -1357,19 +1471,20 @@ cudaError_t launch_batch(const BatchView *d_views, const BatchPlan &P, const Opt
             k_bcolour<<<P.total_colour, kColourThreads, 0, st>>>(d_views, P.cmap, P.gview, t0);
             if (ev) cudaEventRecordWithFlags(ev[6], st, cudaEventRecordExternal);
         }
-        if (P.total_sprep > 0) {
-            const unsigned g = P.total_sprep;
-            if (P.gdim == 2 && col) k_bprep<2, 1, false><<<g, kPrepThreads, sm, st>>>(d_views, P.smap, O, t0);
-            else if (P.gdim == 2) k_bprep<2, 1, true><<<g, kPrepThreads, sm, st>>>(d_views, P.smap, O, t0);
-            else if (col) k_bprep<3, 1, false><<<g, kPrepThreads, sm, st>>>(d_views, P.smap, O, t0);
-            else k_bprep<3, 1, true><<<g, kPrepThreads, sm, st>>>(d_views, P.smap, O, t0);
-        }
-        if (P.total_gprep > 0) {
-            const unsigned g = P.total_gprep;
-            if (P.gdim == 2 && col) k_bprep<2, 2, false><<<g, kPrepThreads, sm, st>>>(d_views, P.gmap, O, t0);
-            else if (P.gdim == 2) k_bprep<2, 2, true><<<g, kPrepThreads, sm, st>>>(d_views, P.gmap, O, t0);
-            else if (col) k_bprep<3, 2, false><<<g, kPrepThreads, sm, st>>>(d_views, P.gmap, O, t0);
-            else k_bprep<3, 2, true><<<g, kPrepThreads, sm, st>>>(d_views, P.gmap, O, t0);
+        // the colours: in the pass above, or here, from staged rows where the
+        // batch's rows allow it
+        const auto prep = [&](auto pass, auto here, auto staged, unsigned g, const int2 *map) {
+            if (g == 0) return;
+            if (col) pass<<<g, kPrepThreads, sm, st>>>(d_views, map, O, t0);
+            else if (P.stage_bytes) staged<<<g, kPrepThreads, stage_smem(P.max_T, P.stage_bytes), st>>>(d_views, map, O, t0);
+            else here<<<g, kPrepThreads, sm, st>>>(d_views, map, O, t0);
+        };
+        if (P.gdim == 2) {
+            prep(k_bprep<2, 1, COL_PASS>, k_bprep<2, 1, COL_HERE>, k_bprep<2, 1, COL_STAGED>, P.total_sprep, P.smap);
+            prep(k_bprep<2, 2, COL_PASS>, k_bprep<2, 2, COL_HERE>, k_bprep<2, 2, COL_STAGED>, P.total_gprep, P.gmap);
+        } else {
+            prep(k_bprep<3, 1, COL_PASS>, k_bprep<3, 1, COL_HERE>, k_bprep<3, 1, COL_STAGED>, P.total_sprep, P.smap);
+            prep(k_bprep<3, 2, COL_PASS>, k_bprep<3, 2, COL_HERE>, k_bprep<3, 2, COL_STAGED>, P.total_gprep, P.gmap);
         }
     }
     mark(1);
@@ -1398,27 +1513,49 @@ cudaError_t launch_batch(const BatchView *d_views, const BatchPlan &P, const Opt
 // (the fill's order CTA needs 64 words)
 size_t local_bins_smem(int T, bool fill) { return fill ? (size_t)(T > 64 ? T : 64) * 4 : (size_t)((T + 1) / 2) * 4; }
 
+// Shared memory of the set-up with staged SH rows.
+static size_t stage_smem(int T, int row_bytes)
+{
+    return (local_bins_smem(T, false) + 15) / 16 * 16 + (size_t)kPrepThreads * row_bytes;
+}
+
+int staged_row_bytes(const SceneView &S, int T)
+{
+    const int row = 3 * kShRows * (S.sh_dtype == GES_F32 ? 4 : 2);
+    const bool aligned = ((reinterpret_cast<uintptr_t>(S.s_sh) | reinterpret_cast<uintptr_t>(S.g_sh)) & 15) == 0;
+    // two CTAs of an SM (1 KB of each is the system's, the batch's keep a view
+    // entry): with one the set-up is slower than with direct loads
+    return S.deg == 3 && aligned && 2 * (stage_smem(T, row) + 2048) <= (size_t)228 * 1024 ? row : 0;
+}
+
 cudaError_t prepare_forward_kernels()
 {
-    cudaError_t e;
-    const int hs = (int)local_bins_smem(kLocalMaxTiles, false);
-    if ((e = cudaFuncSetAttribute(k_prep_local<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, hs)) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(k_prep_local<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, hs)) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(k_prep_local<3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, hs)) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(k_bprep<3, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, hs)) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(k_bprep<3, 2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, hs)) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(k_bprep<2, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, hs)) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(k_bprep<2, 2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, hs)) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(k_bprep<3, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, hs)) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(k_bprep<3, 2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, hs)) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(k_bprep<2, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, hs)) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(k_bprep<2, 2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, hs)) != cudaSuccess)
-        return e;
-    if ((e = cudaFuncSetAttribute(k_fill_local, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)local_bins_smem(kLocalMaxTiles, true))) != cudaSuccess)
-        return e;
-    return cudaFuncSetAttribute(k_bfill, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)local_bins_smem(kLocalMaxTiles, true));
+    const int hs = (int)local_bins_smem(kLocalMaxTiles, false), ss = 113 * 1024;
+    cudaError_t e = cudaSuccess;
+    const auto smem = [&](auto k, int bytes) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    };
+    smem(k_prep_local<3, false, COL_HERE>, hs);
+    smem(k_prep_local<2, false, COL_HERE>, hs);
+    smem(k_prep_local<3, true, COL_HERE>, hs);
+    smem(k_prep_local<3, false, COL_STAGED>, ss);
+    smem(k_prep_local<2, false, COL_STAGED>, ss);
+    smem(k_prep_local<3, true, COL_STAGED>, ss);
+    smem(k_bprep<3, 1, COL_PASS>, hs);
+    smem(k_bprep<3, 2, COL_PASS>, hs);
+    smem(k_bprep<2, 1, COL_PASS>, hs);
+    smem(k_bprep<2, 2, COL_PASS>, hs);
+    smem(k_bprep<3, 1, COL_HERE>, hs);
+    smem(k_bprep<3, 2, COL_HERE>, hs);
+    smem(k_bprep<2, 1, COL_HERE>, hs);
+    smem(k_bprep<2, 2, COL_HERE>, hs);
+    smem(k_bprep<3, 1, COL_STAGED>, ss);
+    smem(k_bprep<3, 2, COL_STAGED>, ss);
+    smem(k_bprep<2, 1, COL_STAGED>, ss);
+    smem(k_bprep<2, 2, COL_STAGED>, ss);
+    smem(k_fill_local, (int)local_bins_smem(kLocalMaxTiles, true));
+    smem(k_bfill, (int)local_bins_smem(kLocalMaxTiles, true));
+    return e;
 }
 
 // Binning through per-CTA histograms; otherwise with global counters.
@@ -1442,9 +1579,14 @@ cudaError_t launch_binning(const SceneView &S, const CamParams &C, const OptPara
         B = plan_local_bins(Sv.N, Sv.M, sms);
         if (B.Ps + B.Pg > 0) {
             const size_t sm = local_bins_smem(T, false);
-            if (X.s_tside) k_prep_local<3, true><<<B.Ps + B.Pg, kPrepThreads, sm, st>>>(Sv, C, O, X, B);
-            else if (Sv.gdim == 2) k_prep_local<2><<<B.Ps + B.Pg, kPrepThreads, sm, st>>>(Sv, C, O, X, B);
-            else k_prep_local<3><<<B.Ps + B.Pg, kPrepThreads, sm, st>>>(Sv, C, O, X, B);
+            const int row = staged_row_bytes(Sv, T);
+            const auto prep = [&](auto here, auto staged) {
+                if (row) staged<<<B.Ps + B.Pg, kPrepThreads, stage_smem(T, row), st>>>(Sv, C, O, X, B);
+                else here<<<B.Ps + B.Pg, kPrepThreads, sm, st>>>(Sv, C, O, X, B);
+            };
+            if (X.s_tside) prep(k_prep_local<3, true, COL_HERE>, k_prep_local<3, true, COL_STAGED>);
+            else if (Sv.gdim == 2) prep(k_prep_local<2, false, COL_HERE>, k_prep_local<2, false, COL_STAGED>);
+            else prep(k_prep_local<3, false, COL_HERE>, k_prep_local<3, false, COL_STAGED>);
         }
     } else {
         const int nsb = (int)((Sv.N + 255) / 256), ngb = (int)((Sv.M + 255) / 256);

@@ -136,6 +136,7 @@ struct BatchPlan {
     int total_sprep, total_gprep;            // preprocess CTAs of the surfel and the Gaussian launch
     int raster_ctas;                         // persistent raster grid
     int gdim;                                // Gaussian kind of every scene (2 or 3; 0 reads as 3)
+    int stage_bytes;                         // SH row bytes the set-up stages in shared memory; 0: direct loads
     // (view, CTA of the view) of each CTA of the surfel / Gaussian preprocess
     // launch: the views of one scene take the same primitive range one after
     // another, so all but the first read its attributes from L2
@@ -163,6 +164,10 @@ constexpr int kAllocTiles = 1024;       // tiles per CTA of the list allocation 
 constexpr int kColTiles = 64;           // tiles per CTA of the column scan
 LocalBins plan_local_bins(int64_t N, int64_t M, int num_sms);
 size_t local_bins_smem(int T, bool fill);
+// SH row bytes of the staged set-up (see sh_stage) for a scene and a number of
+// tiles, or 0 where it does not apply: other degrees, unaligned rows, too many
+// tiles for two CTAs per SM.
+int staged_row_bytes(const SceneView &S, int T);
 cudaError_t prepare_forward_kernels();   // once per device: large dynamic shared memory
 
 // ---------------------------------------------------------------------------
