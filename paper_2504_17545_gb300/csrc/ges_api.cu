@@ -692,12 +692,12 @@ ges_status ges_render_translucent_backward(ges_scene *s, const ges_camera *cam, 
         ges_status r = translucent_setup(s, cam, opts, w, C, O, X);
         if (r != GES_OK) return r;
         const int64_t N = std::max<int64_t>(s->desc.n_surfels, 1);
-        GES_CUDA(s->t_acc.ensure((size_t)N * 18 * 8 + 16));
+        GES_CUDA(s->t_acc.ensure((size_t)N * kTSums * 8 + 16));
         GES_CUDA(cudaMemsetAsync(X.status, 0, ST_WORDS * 4, s->stream));
         long long *acc = (long long *)s->t_acc.p;
         cudaError_t e = launch_translucent_backward(s->view, C, O, X, w, front_first != 0,
                                                     dL_drgb, out_T, out_front,
-                                                    out_last, out_Tlast, acc, (unsigned *)(acc + (size_t)N * 18),
+                                                    out_last, out_Tlast, acc, (unsigned *)(acc + (size_t)N * kTSums),
                                                     grads->s_pos, grads->s_rot, grads->s_scale, grads->s_w,
                                                     grads->s_sh, s->stream);
         if (e != cudaSuccess) return cuda_fail(e, "kernel launch");

@@ -557,8 +557,12 @@ __global__ void __launch_bounds__(kFillThreads, 2) k_fill_local(ViewScratch X, i
                                                              LocalBins B)
 {
     extern __shared__ unsigned cur[];    // T cursors
-    if (blockIdx.x == 0)
-        order_body<false>(X, T, (unsigned long long)X.status[ST_SPAIRS] + X.status[ST_GPAIRS], cur);
+    if (blockIdx.x == 0) {
+        // (the translucent kernels take whole tiles)
+        const unsigned long long total = (unsigned long long)X.status[ST_SPAIRS] + X.status[ST_GPAIRS];
+        if (X.s_tside) order_body<true>(X, T, total, cur);
+        else order_body<false>(X, T, total, cur);
+    }
     else fill_local_body(X, T, tiles_x, tsx, tsy, B, blockIdx.x - 1, cur, X.s_tside != nullptr);
 }
 
@@ -1557,9 +1561,6 @@ cudaError_t prepare_forward_kernels()
     smem(k_bfill, (int)local_bins_smem(kLocalMaxTiles, true));
     return e;
 }
-
-// Binning through per-CTA histograms; otherwise with global counters.
-static bool local_binning(const ViewScratch &X, int T) { return X.hist != nullptr && T <= kLocalMaxTiles; }
 
 // preprocess + binning of one view (everything before the raster)
 cudaError_t launch_binning(const SceneView &S, const CamParams &C, const OptParams &O, const ViewScratch &X,

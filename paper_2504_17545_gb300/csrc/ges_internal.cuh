@@ -168,6 +168,8 @@ size_t local_bins_smem(int T, bool fill);
 // tiles, or 0 where it does not apply: other degrees, unaligned rows, too many
 // tiles for two CTAs per SM.
 int staged_row_bytes(const SceneView &S, int T);
+// Binning through per-CTA histograms; otherwise with global counters.
+inline bool local_binning(const ViewScratch &X, int T) { return X.hist != nullptr && T <= kLocalMaxTiles; }
 cudaError_t prepare_forward_kernels();   // once per device: large dynamic shared memory
 
 // ---------------------------------------------------------------------------
@@ -186,7 +188,8 @@ cudaError_t launch_translucent(const SceneView &S, const CamParams &C, const Opt
                                const float *w, bool front_first, float *out_rgb,
                                float *out_T, int32_t *out_front, int32_t *out_last, float *out_Tlast, int32_t *cover,
                                cudaStream_t st);
-// Its backward: acc [N][18] 64-bit words and gmax (one word) are scratch.
+// Its backward: acc [N][kTSums] 64-bit words and gmax (one word) are scratch.
+constexpr int kTSums = 14;
 cudaError_t launch_translucent_backward(const SceneView &S, const CamParams &C, const OptParams &O,
                                         const ViewScratch &X, const float *w, bool front_first,
                                         const float *dL, const float *in_T,

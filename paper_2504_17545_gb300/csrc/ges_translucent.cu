@@ -17,13 +17,14 @@
 //                sorted order, the frontmost first when front_first is set,
 //                stopping once T < 1e-4 after a blend; C += T bg;
 //   k_tbwd       per pixel in reverse order, dC/dc = alpha T and
-//                dC/dalpha = T (c - S_behind), chained to the surfel's camera-
-//                space frame; the warp reduces each entry's 18 terms in a
-//                fixed order (a halving reduce-scatter) and the lanes holding
-//                the totals add them as 64-bit fixed point, so the result
-//                does not depend on the order of the atomics;
-//   k_tfinal     per surfel: fixed point -> float, camera -> world, rotation
-//                through the quaternion's normalisation, colour -> SH.
+//                dC/dalpha = T (c - S_behind), as moments over the disc; the
+//                warp reduces each entry's 14 terms in a fixed order (a
+//                halving reduce-scatter) and the lanes holding the totals add
+//                them as 64-bit fixed point, so the result does not depend on
+//                the order of the atomics;
+//   k_tfinal     per surfel: fixed point -> float, the moments chained to the
+//                camera-space frame, camera -> world, rotation through the
+//                quaternion's normalisation, colour -> SH.
 #include "ges_internal.cuh"
 
 namespace ges {
@@ -32,7 +33,7 @@ namespace {
 
 constexpr int kSortCap = 4096;          // entries sorted in shared memory
 constexpr float kTStop = 1e-4f;         // blending stops once T falls below this
-constexpr int kTAcc = 18;               // gradient terms accumulated per surfel
+constexpr int kTAcc = kTSums;               // gradient sums per surfel (see t_terms)
 
 __device__ __forceinline__ unsigned lane_idx() { return threadIdx.x & 31u; }
 
@@ -60,18 +61,98 @@ __device__ __forceinline__ void bitonic(unsigned long long *a, int n, int m)
     }
 }
 
+// Ascending bitonic sort of 256 kE keys, kE consecutive ones per thread, up to
+// runs of m keys (a power of two >= kE).  Partners fewer than kE apart are in
+// the thread's registers, fewer than 32 kE apart in its warp (shuffles); only
+// larger steps go through shared memory, 6 of the 45 of a 512-key sort.  With
+// every step in shared memory behind a barrier the sort of a 1080p view's
+// lists (2.0M keys) took 118 us, this 71.
+template <int kE>
+__device__ __forceinline__ void sort_regs(unsigned long long (&v)[kE], unsigned long long *sk, int m)
+{
+    const int t = threadIdx.x;
+    const auto keep = [](unsigned long long a, unsigned long long b, bool low) { return (a < b) == low ? a : b; };
+    // partner thread t ^ x, its element e ^ f; the lower index keeps the smaller key
+    const auto step = [&](int x, int f, bool low) {
+        unsigned long long o[kE];
+        if (x < 32) {
+#pragma unroll
+            for (int e = 0; e < kE; ++e) o[e] = __shfl_xor_sync(0xffffffffu, v[e], x);
+        } else {
+            __syncthreads();
+#pragma unroll
+            for (int e = 0; e < kE; ++e) sk[e * 256 + t] = v[e];
+            __syncthreads();
+#pragma unroll
+            for (int e = 0; e < kE; ++e) o[e] = sk[e * 256 + (t ^ x)];
+        }
+        unsigned long long n[kE];
+#pragma unroll
+        for (int e = 0; e < kE; ++e) n[e] = keep(v[e], f ? o[kE - 1 - e] : o[e], low);
+#pragma unroll
+        for (int e = 0; e < kE; ++e) v[e] = n[e];
+    };
+    const auto inside = [&](int e, int o) {
+        const unsigned long long a = v[e], b = v[o];
+        v[e] = a < b ? a : b;
+        v[o] = a < b ? b : a;
+    };
+    for (int k = 2; k <= m; k <<= 1) {
+        // merge runs of k / 2: against the reversed neighbour, then halving distances
+        if (k <= kE) {
+#pragma unroll
+            for (int kk = 2; kk <= kE; kk <<= 1)
+                if (kk == k) {
+#pragma unroll
+                    for (int e = 0; e < kE; ++e)
+                        if ((e & (kk >> 1)) == 0) inside(e, e ^ (kk - 1));
+                }
+        } else {
+            const int x = k / kE - 1;
+            step(x, 1, (t & ((x + 1) >> 1)) == 0);
+        }
+        for (int j = k >> 2; j >= kE; j >>= 1) step(j / kE, 0, (t & (j / kE)) == 0);
+#pragma unroll
+        for (int j = kE >> 1; j >= 1; j >>= 1)
+            if (j <= k >> 2) {
+#pragma unroll
+                for (int e = 0; e < kE; ++e)
+                    if ((e & j) == 0) inside(e, e ^ j);
+            }
+    }
+}
+
+template <int kE>
+__device__ __forceinline__ void sort_tile(unsigned long long *keys, int n, int m, unsigned long long *sk)
+{
+    unsigned long long v[kE];
+#pragma unroll
+    for (int e = 0; e < kE; ++e) v[e] = kE * (int)threadIdx.x + e < n ? keys[kE * threadIdx.x + e] : ~0ull;
+    sort_regs<kE>(v, sk, m < kE ? kE : m);
+#pragma unroll
+    for (int e = 0; e < kE; ++e)
+        if (kE * (int)threadIdx.x + e < n) keys[kE * threadIdx.x + e] = v[e];
+}
+
 // The list entries are the sort keys: (id, depth key) read as one 64-bit word
 // with the depth key above.
-__global__ void __launch_bounds__(256) k_tsort(const int2 *__restrict__ rng, uint2 *list, const unsigned *status)
+__global__ void __launch_bounds__(256) k_tsort(ViewScratch X)
 {
     __shared__ unsigned long long sk[kSortCap];
-    if (status[ST_FLAGS] & FLAG_SOVF) return;
-    const int a = rng[blockIdx.x].x, n = rng[blockIdx.x].y - a;
+    if (X.status[ST_FLAGS] & FLAG_SOVF) return;
+    const int2 rng = X.s_rng[X.order ? X.order[blockIdx.x] : blockIdx.x];
+    const int a = rng.x, n = rng.y - a;
     if (n <= 1) return;
-    unsigned long long *keys = reinterpret_cast<unsigned long long *>(list) + a;
+    unsigned long long *keys = reinterpret_cast<unsigned long long *>(X.s_list) + a;
     int m = 1;
     while (m < n) m <<= 1;
-    if (n <= kSortCap) {
+    if (n <= 256) {
+        sort_tile<1>(keys, n, m, sk);
+    } else if (n <= 512) {
+        sort_tile<2>(keys, n, m, sk);
+    } else if (n <= 1024) {
+        sort_tile<4>(keys, n, m, sk);
+    } else if (n <= kSortCap) {
         for (int k = threadIdx.x; k < n; k += blockDim.x) sk[k] = keys[k];
         __syncthreads();
         bitonic(sk, n, m);
@@ -132,7 +213,7 @@ __global__ void __launch_bounds__(kRasterThreads, 4)
     __shared__ float sizmax[kRasterThreads];
     __shared__ float slw[kRasterThreads];        // log w
     if (X.status[ST_FLAGS] & FLAG_SOVF) return;
-    const int tile = blockIdx.x, tx = tile % C.tiles_x, ty = tile / C.tiles_x;
+    const int tile = X.order ? (int)X.order[blockIdx.x] : (int)blockIdx.x, tx = tile % C.tiles_x, ty = tile / C.tiles_x;
     const unsigned warp = threadIdx.x >> 5, lane = lane_idx();
     const int wx0 = tx * kTile + (warp & 1) * kWarpW, wy0 = ty * kTile + (warp >> 1) * kWarpH;
     const int wx1 = min(wx0 + kWarpW - 1, C.W - 1), wy1 = min(wy0 + kWarpH - 1, C.H - 1);
@@ -251,54 +332,60 @@ __global__ void __launch_bounds__(kRasterThreads, 4)
     if (cover && has_front) atomicAdd(cover + fid, 1);
 }
 
-// the 18 per-(pixel, surfel) gradient terms: gP(3) gU(3) gV(3) gN(3) gs1 gs2 gw gc(3), camera space
+// The sums of one (pixel, surfel): dL/dc (3), dL/dw, and what every geometry
+// gradient is a linear combination of: with rho' = dL/d(a^2 + b^2) and
+// h = 2 rho' (a U.d/s1 + b V.d/s2) / N.d (the hit moving along the ray d),
+//   rho' {a, b, a^2, ab, b^2},  h {1, a, b},
+// and rho' {a/s1, b/s2} 2 X.N: the hit X = z d - P lies in the plane but for its
+// rounding, which the rotation's gradient sees (leaving it out moved single
+// gradients by 6e-4 of their root mean square).  The frame and the scales enter once per surfel, in k_tfinal.  Summing the 14
+// gradients of position, frame and scales themselves took twice the
+// instructions per pair (and 18 sums to reduce and to add instead of 14):
+// k_tbwd 323 -> 239 us at 1080p, 1M surfels, front first (at 3 CTAs per SM 274).
+// fr: the surfel's camera-space frame (P, s1), (U, s2), (V, -), (N, -).
 __device__ __forceinline__ void t_terms(const float4 *fr, float a, float G, float wv, float T, float iz,
                                         const float *g, const float *cS, const float *col, float u, float v,
                                         const CamParams &C, float *out)
 {
     float dLda = 0.f;
     for (int ch = 0; ch < 3; ++ch) {
-        out[15 + ch] = a * T * g[ch];
+        out[ch] = a * T * g[ch];
         dLda += T * (col[ch] - cS[ch]) * g[ch];
     }
-    for (int k = 0; k < 15; ++k) out[k] = 0.f;
-    if (!(wv * G < 1.f)) return;                    // alpha clamped at 1: no geometry gradient
-    out[14] = dLda * G;
-    const float dLdrho = dLda * (-0.5f * wv * G);
-    const float4 f0 = fr[0], f1 = fr[1], f2 = fr[2], f3 = fr[3];
-    const float P[3] = {f0.x, f0.y, f0.z}, U[3] = {f1.x, f1.y, f1.z}, V[3] = {f2.x, f2.y, f2.z};
-    const float Nn[3] = {f3.x, f3.y, f3.z}, s1 = f0.w, s2 = f1.w;
-    const float d[3] = {(u - C.cx) / C.fx, (v - C.cy) / C.fy, 1.f};
-    const float Nd = Nn[0] * d[0] + Nn[1] * d[1] + Nn[2] * d[2];
-    const float Ud = U[0] * d[0] + U[1] * d[1] + U[2] * d[2];
-    const float Vd = V[0] * d[0] + V[1] * d[1] + V[2] * d[2];
-    const float z = 1.f / iz;
-    float Xv[3];
-    for (int q = 0; q < 3; ++q) Xv[q] = z * d[q] - P[q];
-    const float aa = (Xv[0] * U[0] + Xv[1] * U[1] + Xv[2] * U[2]) / s1;
-    const float bb = (Xv[0] * V[0] + Xv[1] * V[1] + Xv[2] * V[2]) / s2;
-    const float dLa = dLdrho * 2.f * aa, dLb = dLdrho * 2.f * bb;
-    for (int q = 0; q < 3; ++q) {
-        out[q] = dLa * ((Ud / Nd) * Nn[q] - U[q]) / s1 + dLb * ((Vd / Nd) * Nn[q] - V[q]) / s2;
-        out[3 + q] = dLa * Xv[q] / s1;
-        out[6 + q] = dLb * Xv[q] / s2;
-        out[9 + q] = -(dLa * Ud / s1 + dLb * Vd / s2) * Xv[q] / Nd;
-    }
-    out[12] = dLa * (-aa / s1);
-    out[13] = dLb * (-bb / s2);
+    const bool free_ = wv * G < 1.f;                // clamped at 1: no gradient but the colour's
+    out[3] = free_ ? dLda * G : 0.f;
+    const float rp = free_ ? dLda * (-0.5f * wv * G) : 0.f;
+    const float4 f0 = __ldg(fr), f1 = __ldg(fr + 1), f2 = __ldg(fr + 2), f3 = __ldg(fr + 3);
+    const float z = 1.f / iz, d0 = (u - C.cx) / C.fx, d1 = (v - C.cy) / C.fy;
+    const float X0 = z * d0 - f0.x, X1 = z * d1 - f0.y, X2 = z - f0.z;
+    const float aa = (X0 * f1.x + X1 * f1.y + X2 * f1.z) / f0.w, bb = (X0 * f2.x + X1 * f2.y + X2 * f2.z) / f1.w;
+    const float Ud = f1.x * d0 + f1.y * d1 + f1.z, Vd = f2.x * d0 + f2.y * d1 + f2.z;
+    const float Nd = f3.x * d0 + f3.y * d1 + f3.z;
+    const float ra = rp * aa, rb = rp * bb;
+    const float h = 2.f * (ra * Ud / f0.w + rb * Vd / f1.w) / Nd;
+    out[4] = ra;
+    out[5] = rb;
+    out[6] = ra * aa;
+    out[7] = ra * bb;
+    out[8] = rb * bb;
+    out[9] = h;
+    out[10] = h * aa;
+    out[11] = h * bb;
+    const float xn = 2.f * (X0 * f3.x + X1 * f3.y + X2 * f3.z);
+    out[12] = ra * xn / f0.w;
+    out[13] = rb * xn / f1.w;
 }
 
-__device__ __forceinline__ void t_add(long long *acc, int id, const float *terms, float scale)
+// Sum k in units of max |dL/dC| 2^-30 (the sums of h, which grow with 1/s and
+// 1/N.d: 2^-24), as an integer (the fast conversion holds below 2^42).
+__device__ __forceinline__ constexpr float t_units(int k) { return k < 9 ? 1073741824.f : 16777216.f; }
+__device__ __forceinline__ void t_add(unsigned long long *a, float x)
 {
-    long long *a = acc + (int64_t)kTAcc * id;
-    for (int k = 0; k < kTAcc; ++k) {
-        const float x = terms[k] * scale;
-        if (x != 0.f) atomicAdd(reinterpret_cast<unsigned long long *>(a + k), (unsigned long long)__float2ll_rn(x));
-    }
+    if (x != 0.f) atomicAdd(a, (unsigned long long)(fabsf(x) < 4398046511104.f ? f2ll_rn(x) : __float2ll_rn(x)));
 }
 
 template <bool kFront>
-__global__ void __launch_bounds__(kRasterThreads, 3)
+__global__ void __launch_bounds__(kRasterThreads, 4)
     k_tbwd(ViewScratch X, CamParams C, OptParams O, const float *__restrict__ w, const float *__restrict__ dL,
            const float *__restrict__ in_T, const int32_t *__restrict__ in_front, const int32_t *__restrict__ in_last,
            const float *__restrict__ in_Tlast, const unsigned *gmax_bits, long long *acc)
@@ -312,8 +399,8 @@ __global__ void __launch_bounds__(kRasterThreads, 3)
     if (X.status[ST_FLAGS] & FLAG_SOVF) return;
     const float gmax = __uint_as_float(*gmax_bits);
     if (!(gmax > 0.f)) return;
-    const float scale = 16777216.f / gmax;        // 2^24 / max |dL/dC|
-    const int tile = blockIdx.x, tx = tile % C.tiles_x, ty = tile / C.tiles_x;
+    const float scale = 1.f / gmax;
+    const int tile = X.order ? (int)X.order[blockIdx.x] : (int)blockIdx.x, tx = tile % C.tiles_x, ty = tile / C.tiles_x;
     const unsigned warp = threadIdx.x >> 5, lane = lane_idx();
     const int wx0 = tx * kTile + (warp & 1) * kWarpW, wy0 = ty * kTile + (warp >> 1) * kWarpH;
     const int wx1 = min(wx0 + kWarpW - 1, C.W - 1), wy1 = min(wy0 + kWarpH - 1, C.H - 1);
@@ -388,11 +475,10 @@ __global__ void __launch_bounds__(kRasterThreads, 3)
                 if (!__any_sync(0xffffffffu, contrib)) continue;
                 if (!contrib)
                     for (int k = 0; k < kTAcc; ++k) terms[k] = 0.f;
-                // the warp's 18 sums, each added by the lane that ends up holding it
+                // the warp's sums, each added by the lane that ends up holding it
                 unsigned long long *ak = reinterpret_cast<unsigned long long *>(acc + (int64_t)kTAcc * id);
                 warp_reduce_scatter<kTAcc>(terms, (int)lane, [&](int k, float tot) {
-                    const float x = tot * scale;
-                    if (x != 0.f) atomicAdd(ak + k, (unsigned long long)__float2ll_rn(x));
+                    t_add(ak + k, tot * (t_units(k) * scale));
                 });
             }
         }
@@ -407,23 +493,25 @@ __global__ void __launch_bounds__(kRasterThreads, 3)
             float terms[kTAcc];
             t_terms(X.s_tside + 4 * (int64_t)myfront, a, G, w[myfront], !first_seen ? Tl : 1.f, iz, g, S, col, u, v,
                     C, terms);
-            t_add(acc, myfront, terms, scale);
+            unsigned long long *ak = reinterpret_cast<unsigned long long *>(acc + (int64_t)kTAcc * myfront);
+            for (int k = 0; k < kTAcc; ++k) t_add(ak + k, terms[k] * (t_units(k) * scale));
         }
     }
 }
 
 // per surfel: fixed point -> float, camera -> world, rotation through the
 // quaternion's normalisation, colour -> SH (and position through the view direction)
-__global__ void __launch_bounds__(256) k_tfinal(SceneView S, CamParams C, const long long *__restrict__ acc,
+__global__ void __launch_bounds__(256) k_tfinal(SceneView S, CamParams C, const float4 *__restrict__ tside,
+                                                const long long *__restrict__ acc,
                                                 const unsigned *gmax_bits, float *g_pos, float *g_rot,
                                                 float *g_scale, float *g_w, float *g_sh)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= S.N) return;
     const float gm = __uint_as_float(*gmax_bits);
-    const float inv = gm > 0.f ? gm / 16777216.f : 0.f;
     float A[kTAcc];
-    for (int k = 0; k < kTAcc; ++k) A[k] = (float)acc[(int64_t)kTAcc * i + k] * inv;
+    for (int k = 0; k < kTAcc; ++k)
+        A[k] = gm > 0.f ? __ll2float_rn(__ldg(acc + (int64_t)kTAcc * i + k)) * (gm / t_units(k)) : 0.f;
     const int K = (S.deg + 1) * (S.deg + 1);
     bool any = false;
     for (int k = 0; k < kTAcc; ++k) any |= A[k] != 0.f;
@@ -439,10 +527,24 @@ __global__ void __launch_bounds__(256) k_tfinal(SceneView S, CamParams C, const 
     float q[4], R[9], qn[4], qnorm;
     for (int k = 0; k < 4; ++k) q[k] = load_attr(S.s_rot, 4 * i + k, S.attr_dtype);
     const bool okq = quat_to_rot(q[0], q[1], q[2], q[3], R, qn, &qnorm);
+    // the sums and the set-up's camera-space frame: the chain rule of a = X.U/s1,
+    // b = X.V/s2 with the hit X = a s1 U + b s2 V relative to the centre
+    const float4 f0 = __ldg(tside + 4 * i), f1 = __ldg(tside + 4 * i + 1), f2 = __ldg(tside + 4 * i + 2);
+    const float4 f3 = __ldg(tside + 4 * i + 3);
+    const float U[3] = {f1.x, f1.y, f1.z}, V[3] = {f2.x, f2.y, f2.z}, Nn[3] = {f3.x, f3.y, f3.z};
+    const float s1 = f0.w, s2 = f1.w;
+    const float Sa = A[4], Sb = A[5], Saa = A[6], Sab = A[7], Sbb = A[8], Sh = A[9], Sha = A[10], Shb = A[11];
+    float gP[3], gU[3], gV[3], gN[3];
+    for (int q = 0; q < 3; ++q) {
+        gP[q] = Nn[q] * Sh - U[q] * (2.f * Sa / s1) - V[q] * (2.f * Sb / s2);
+        gU[q] = 2.f * (Saa * U[q] + (s2 / s1) * Sab * V[q]) + A[12] * Nn[q];
+        gV[q] = 2.f * ((s1 / s2) * Sab * U[q] + Sbb * V[q]) + A[13] * Nn[q];
+        gN[q] = -(s1 * Sha * U[q] + s2 * Shb * V[q]);
+    }
     float gp[3];
-    for (int a = 0; a < 3; ++a) gp[a] = C.R[a] * A[0] + C.R[3 + a] * A[1] + C.R[6 + a] * A[2];
-    if (g_scale) { g_scale[2 * i] = A[12]; g_scale[2 * i + 1] = A[13]; }
-    if (g_w) g_w[i] = A[14];
+    for (int a = 0; a < 3; ++a) gp[a] = C.R[a] * gP[0] + C.R[3 + a] * gP[1] + C.R[6 + a] * gP[2];
+    if (g_scale) { g_scale[2 * i] = -2.f * Saa / s1; g_scale[2 * i + 1] = -2.f * Sbb / s2; }
+    if (g_w) g_w[i] = A[3];
     // colour -> SH coefficients and position (through the view direction)
     float dir[3], dist;
     view_dir(C, __ldg(S.s_pos + 3 * i), __ldg(S.s_pos + 3 * i + 1), __ldg(S.s_pos + 3 * i + 2), dir, dist);
@@ -451,7 +553,7 @@ __global__ void __launch_bounds__(256) k_tfinal(SceneView S, CamParams C, const 
     float rgb[3], raw[3];
     sh_colour(S.s_sh, i, K, S.sh_dtype, Y, rgb, raw);
     float gc[3];
-    for (int c = 0; c < 3; ++c) gc[c] = raw[c] > 0.f ? A[15 + c] : 0.f;
+    for (int c = 0; c < 3; ++c) gc[c] = raw[c] > 0.f ? A[c] : 0.f;
     float gd[3] = {0.f, 0.f, 0.f};
     switch (K) {
     case 16: sh_weighted_grad<16>(S.s_sh, i, S.sh_dtype, gc, dir, gd); break;
@@ -470,9 +572,9 @@ __global__ void __launch_bounds__(256) k_tfinal(SceneView S, CamParams C, const 
     // dL/dR[:,k] = Rc^T g_{U,V,N}
     float GR[3][3];
     for (int a = 0; a < 3; ++a) {
-        GR[a][0] = C.R[a] * A[3] + C.R[3 + a] * A[4] + C.R[6 + a] * A[5];
-        GR[a][1] = C.R[a] * A[6] + C.R[3 + a] * A[7] + C.R[6 + a] * A[8];
-        GR[a][2] = C.R[a] * A[9] + C.R[3 + a] * A[10] + C.R[6 + a] * A[11];
+        GR[a][0] = C.R[a] * gU[0] + C.R[3 + a] * gU[1] + C.R[6 + a] * gU[2];
+        GR[a][1] = C.R[a] * gV[0] + C.R[3 + a] * gV[1] + C.R[6 + a] * gV[2];
+        GR[a][2] = C.R[a] * gN[0] + C.R[3 + a] * gN[1] + C.R[6 + a] * gN[2];
     }
     const float wq = qn[0], qx = qn[1], qy = qn[2], qz = qn[3];
     float gq[4];
@@ -562,24 +664,26 @@ __global__ void __launch_bounds__(256) k_contrib(SceneView S, CamParams C, OptPa
 
 }  // namespace
 
-cudaError_t launch_translucent(const SceneView &S, const CamParams &C, const OptParams &O, const ViewScratch &X,
+cudaError_t launch_translucent(const SceneView &S, const CamParams &C, const OptParams &O, const ViewScratch &Xs,
                                const float *w, bool front_first, float *out_rgb,
                                float *out_T, int32_t *out_front, int32_t *out_last, float *out_Tlast, int32_t *cover,
                                cudaStream_t st)
 {
     OptParams Os = O;
     Os.mode = GES_MODE_SURFELS_ONLY;
+    const int T = C.tiles_x * C.tiles_y;
+    ViewScratch X = Xs;
+    if (!local_binning(X, T)) X.order = nullptr;
     cudaError_t e = launch_binning(S, C, Os, X, st, nullptr);
     if (e != cudaSuccess) return e;
-    const int T = C.tiles_x * C.tiles_y;
-    k_tsort<<<T, 256, 0, st>>>(X.s_rng, X.s_list, X.status);
+    k_tsort<<<T, 256, 0, st>>>(X);
     if (front_first) k_traster<true><<<T, kRasterThreads, 0, st>>>(X, C, Os, w, out_rgb, out_T, out_front, out_last, out_Tlast, cover);
     else k_traster<false><<<T, kRasterThreads, 0, st>>>(X, C, Os, w, out_rgb, out_T, out_front, out_last, out_Tlast, cover);
     return cudaGetLastError();
 }
 
 cudaError_t launch_translucent_backward(const SceneView &S, const CamParams &C, const OptParams &O,
-                                        const ViewScratch &X, const float *w, bool front_first,
+                                        const ViewScratch &Xs, const float *w, bool front_first,
                                         const float *dL, const float *in_T,
                                         const int32_t *in_front, const int32_t *in_last, const float *in_Tlast,
                                         long long *acc, unsigned *gmax, float *g_pos, float *g_rot, float *g_scale,
@@ -588,17 +692,19 @@ cudaError_t launch_translucent_backward(const SceneView &S, const CamParams &C, 
     OptParams Os = O;
     Os.mode = GES_MODE_SURFELS_ONLY;
     // the same binning and order as the forward pass (both are deterministic)
+    const int T = C.tiles_x * C.tiles_y;
+    ViewScratch X = Xs;
+    if (!local_binning(X, T)) X.order = nullptr;
     cudaError_t e = launch_binning(S, C, Os, X, st, nullptr);
     if (e != cudaSuccess) return e;
-    const int T = C.tiles_x * C.tiles_y;
-    k_tsort<<<T, 256, 0, st>>>(X.s_rng, X.s_list, X.status);
+    k_tsort<<<T, 256, 0, st>>>(X);
     if ((e = cudaMemsetAsync(acc, 0, sizeof(long long) * kTAcc * (size_t)(S.N > 0 ? S.N : 1), st)) != cudaSuccess)
         return e;
     if ((e = launch_absmax(dL, 3 * (int64_t)C.W * C.H, gmax, st)) != cudaSuccess) return e;
     if (front_first) k_tbwd<true><<<T, kRasterThreads, 0, st>>>(X, C, Os, w, dL, in_T, in_front, in_last, in_Tlast, gmax, acc);
     else k_tbwd<false><<<T, kRasterThreads, 0, st>>>(X, C, Os, w, dL, in_T, in_front, in_last, in_Tlast, gmax, acc);
     if (S.N > 0)
-        k_tfinal<<<(unsigned)((S.N + 255) / 256), 256, 0, st>>>(S, C, acc, gmax, g_pos, g_rot, g_scale, g_w, g_sh);
+        k_tfinal<<<(unsigned)((S.N + 255) / 256), 256, 0, st>>>(S, C, X.s_tside, acc, gmax, g_pos, g_rot, g_scale, g_w, g_sh);
     return cudaGetLastError();
 }
 
