@@ -311,10 +311,10 @@ __global__ void __launch_bounds__(256, 4) k_gbwd_sweep(int64_t M, CamParams C, O
     }
 }
 
-// Colour -> SH coefficients (stored) and position through the view direction
-// (added to gp).
+// Colour -> SH coefficients (their factors left in slot) and position through
+// the view direction (added to gp).
 __device__ __forceinline__ void colour_grad(const SceneView &S, int64_t gi, int K, const GaussOut &o,
-                                            const float *dc, const ges_grads &G, float *gp)
+                                            const float *dc, const ges_grads &G, float *slot, float *gp)
 {
     float Y[16];
     sh_basis(K, o.dir[0], o.dir[1], o.dir[2], Y);
@@ -327,7 +327,7 @@ __device__ __forceinline__ void colour_grad(const SceneView &S, int64_t gi, int 
     case 4: sh_weighted_grad<4>(S.g_sh, gi, S.sh_dtype, gc, o.dir, gd); break;
     default: break;   // degree 0: the colour does not depend on the direction
     }
-    if (G.g_sh) store_sh_grad(G.g_sh + 3 * K * gi, K, Y, gc, nullptr);
+    if (G.g_sh) put_sh_row(slot, K, Y, gc, nullptr);
     if (o.dist > 0.f) {
         const float pr = gd[0] * o.dir[0] + gd[1] * o.dir[1] + gd[2] * o.dir[2];
         for (int a = 0; a < 3; ++a) gp[a] -= (gd[a] - pr * o.dir[a]) / o.dist;
@@ -358,12 +358,10 @@ __device__ __forceinline__ void rot_grad(const float (*GR)[3], const GaussOut &o
     }
 }
 
-__global__ void __launch_bounds__(256, 3) k_gbwd_chain(SceneView S, CamParams C, OptParams O,
-                                                   const float *__restrict__ sums,
-                                                   const float *__restrict__ chain, ges_grads G)
+__device__ __forceinline__ void gbwd_chain(const SceneView &S, const CamParams &C, const OptParams &O, int64_t gi,
+                                         const float *__restrict__ sums, const float *__restrict__ chain,
+                                         const ges_grads &G, float *slot)
 {
-    const int64_t gi = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    if (gi >= S.M) return;
     const int K = (S.deg + 1) * (S.deg + 1);
     unsigned bits = 0u;
     for (int c = 0; c < 9; ++c) bits |= __float_as_uint(__ldg(sums + (int64_t)c * S.M + gi)) & 0x7fffffffu;
@@ -380,14 +378,14 @@ __global__ void __launch_bounds__(256, 3) k_gbwd_chain(SceneView S, CamParams C,
         if (G.g_rot) for (int a = 0; a < 4; ++a) G.g_rot[4 * gi + a] = 0.f;
         if (G.g_scale) for (int a = 0; a < 3; ++a) G.g_scale[3 * gi + a] = 0.f;
         if (G.g_opac) G.g_opac[gi] = 0.f;
-        if (G.g_sh) store_zeros(G.g_sh + 3 * K * gi, 3 * K);
+        if (G.g_sh) put_sh_zeros(slot);
         return;
     }
     float my[9];
     for (int c = 0; c < 9; ++c) my[c] = sums[(int64_t)c * S.M + gi];
     const float *dc = my;
     float gp[3] = {0.f, 0.f, 0.f};
-    colour_grad(S, gi, K, o, dc, G, gp);
+    colour_grad(S, gi, K, o, dc, G, slot, gp);
     // my[3] is dL/dsigma with sigma = sigma0 k3 k2 (the Mip-GES factors, 1 without them)
     if (G.g_opac) G.g_opac[gi] = my[3] * o.k3 * o.k2;
     // conic Q = Sigma2^-1:  dL/dSigma2 = -Q GQ Q with GQ = [[dia, dib/2], [dib/2, dic]]
@@ -467,15 +465,23 @@ __global__ void __launch_bounds__(256, 3) k_gbwd_chain(SceneView S, CamParams C,
     if (G.g_scale) for (int b = 0; b < 3; ++b) G.g_scale[3 * gi + b] = gsc[b];
     if (G.g_rot) rot_grad(GR, o, G.g_rot, gi);
 }
+__global__ void __launch_bounds__(256, 3) k_gbwd_chain(SceneView S, CamParams C, OptParams O,
+                                                   const float *__restrict__ sums,
+                                                   const float *__restrict__ chain, ges_grads G)
+{
+    __shared__ float slots[256 * kShSlot];
+    const int64_t gi = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (gi < S.M) gbwd_chain(S, C, O, gi, sums, chain, G, slots + kShSlot * threadIdx.x);
+    if (G.g_sh)
+        flush_sh_rows(G.g_sh, gi & ~(int64_t)31, S.M, (S.deg + 1) * (S.deg + 1), slots + kShSlot * (threadIdx.x & ~31u));
+}
 
 // 2D Gaussians: the chain rule from the 11 sums of the sweep (dc, dL/dalpha
 // alpha, the seven moments of rho') and the kept set-up words.
-__global__ void __launch_bounds__(256, 3) k_gbwd_chain2(SceneView S, CamParams C, OptParams O,
-                                                    const float *__restrict__ sums,
-                                                    const float *__restrict__ chain, ges_grads G)
+__device__ __forceinline__ void gbwd_chain2(const SceneView &S, const CamParams &C, const OptParams &O, int64_t gi,
+                                         const float *__restrict__ sums, const float *__restrict__ chain,
+                                         const ges_grads &G, float *slot)
 {
-    const int64_t gi = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    if (gi >= S.M) return;
     const int K = (S.deg + 1) * (S.deg + 1);
     float my[11];
     unsigned bits = 0u;
@@ -488,7 +494,7 @@ __global__ void __launch_bounds__(256, 3) k_gbwd_chain2(SceneView S, CamParams C
         if (G.g_rot) for (int a = 0; a < 4; ++a) G.g_rot[4 * gi + a] = 0.f;
         if (G.g_scale) for (int a = 0; a < 2; ++a) G.g_scale[2 * gi + a] = 0.f;
         if (G.g_opac) G.g_opac[gi] = 0.f;
-        if (G.g_sh) store_zeros(G.g_sh + 3 * K * gi, 3 * K);
+        if (G.g_sh) put_sh_zeros(slot);
         return;
     }
     GaussOut o;
@@ -506,7 +512,7 @@ __global__ void __launch_bounds__(256, 3) k_gbwd_chain2(SceneView S, CamParams C
     for (int k = 0; k < 3; ++k) o.raw[k] = v[f++];
 
     float gp[3] = {0.f, 0.f, 0.f};
-    colour_grad(S, gi, K, o, my, G, gp);
+    colour_grad(S, gi, K, o, my, G, slot, gp);
     // sigma' = sigma0 / (S1 S2): dalpha/dsigma' = alpha / sigma'
     const float sigp = sigma0 / (S1 * S2);
     const float dsig = my[3] / sigp;
@@ -581,6 +587,16 @@ __global__ void __launch_bounds__(256, 3) k_gbwd_chain2(SceneView S, CamParams C
     if (G.g_pos) for (int a = 0; a < 3; ++a) G.g_pos[3 * gi + a] = gp[a];
     if (G.g_rot) rot_grad(GR, o, G.g_rot, gi);
 }
+__global__ void __launch_bounds__(256, 3) k_gbwd_chain2(SceneView S, CamParams C, OptParams O,
+                                                   const float *__restrict__ sums,
+                                                   const float *__restrict__ chain, ges_grads G)
+{
+    __shared__ float slots[256 * kShSlot];
+    const int64_t gi = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (gi < S.M) gbwd_chain2(S, C, O, gi, sums, chain, G, slots + kShSlot * threadIdx.x);
+    if (G.g_sh)
+        flush_sh_rows(G.g_sh, gi & ~(int64_t)31, S.M, (S.deg + 1) * (S.deg + 1), slots + kShSlot * (threadIdx.x & ~31u));
+}
 
 // largest |x| (non-negative floats order like their bit patterns)
 __global__ void __launch_bounds__(256) k_absmax(const float *__restrict__ x, int64_t n, unsigned *out)
@@ -639,22 +655,24 @@ __global__ void __launch_bounds__(256) k_surfel_scatter(int64_t N, CamParams C, 
 __global__ void __launch_bounds__(256) k_surfel_sh(SceneView S, CamParams C, const long long *__restrict__ acc,
                                                   const unsigned *__restrict__ gmax_bits, float *__restrict__ g_sh)
 {
+    __shared__ float slots[256 * kShSlot];
     const int64_t si = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    if (si >= S.N) return;
     const int K = (S.deg + 1) * (S.deg + 1);
-    float *out = g_sh + (int64_t)3 * K * si;
-    const long long a0 = acc[3 * si], a1 = acc[3 * si + 1], a2 = acc[3 * si + 2];
+    float *slot = slots + kShSlot * threadIdx.x;
+    long long a0 = 0, a1 = 0, a2 = 0;
+    if (si < S.N) { a0 = acc[3 * si]; a1 = acc[3 * si + 1]; a2 = acc[3 * si + 2]; }
     if (a0 == 0 && a1 == 0 && a2 == 0) {
-        store_zeros(out, 3 * K);
-        return;
+        put_sh_zeros(slot);
+    } else {
+        const float unit = __uint_as_float(*gmax_bits) * 9.31322574615478516e-10f;   // gmax 2^-30
+        const float gc[3] = {__ll2float_rn(a0) * unit, __ll2float_rn(a1) * unit, __ll2float_rn(a2) * unit};
+        float dir[3], L, Y[16], rgb[3], raw[3];
+        view_dir(C, __ldg(S.s_pos + 3 * si), __ldg(S.s_pos + 3 * si + 1), __ldg(S.s_pos + 3 * si + 2), dir, L);
+        sh_basis(K, dir[0], dir[1], dir[2], Y);
+        sh_colour(S.s_sh, si, K, S.sh_dtype, Y, rgb, raw);
+        put_sh_row(slot, K, Y, gc, raw);
     }
-    const float unit = __uint_as_float(*gmax_bits) * 9.31322574615478516e-10f;   // gmax 2^-30
-    const float gc[3] = {__ll2float_rn(a0) * unit, __ll2float_rn(a1) * unit, __ll2float_rn(a2) * unit};
-    float dir[3], L, Y[16], rgb[3], raw[3];
-    view_dir(C, __ldg(S.s_pos + 3 * si), __ldg(S.s_pos + 3 * si + 1), __ldg(S.s_pos + 3 * si + 2), dir, L);
-    sh_basis(K, dir[0], dir[1], dir[2], Y);
-    sh_colour(S.s_sh, si, K, S.sh_dtype, Y, rgb, raw);
-    store_sh_grad(out, K, Y, gc, raw);
+    flush_sh_rows(g_sh, si & ~(int64_t)31, S.N, K, slots + kShSlot * (threadIdx.x & ~31u));
 }
 
 }  // namespace

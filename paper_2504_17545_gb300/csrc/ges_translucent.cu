@@ -501,13 +501,11 @@ __global__ void __launch_bounds__(kRasterThreads, 4)
 
 // per surfel: fixed point -> float, camera -> world, rotation through the
 // quaternion's normalisation, colour -> SH (and position through the view direction)
-__global__ void __launch_bounds__(256) k_tfinal(SceneView S, CamParams C, const float4 *__restrict__ tside,
-                                                const long long *__restrict__ acc,
-                                                const unsigned *gmax_bits, float *g_pos, float *g_rot,
-                                                float *g_scale, float *g_w, float *g_sh)
+__device__ __forceinline__ void tfinal(const SceneView &S, const CamParams &C, int64_t i,
+                                       const float4 *__restrict__ tside, const long long *__restrict__ acc,
+                                       const unsigned *gmax_bits, float *g_pos, float *g_rot, float *g_scale,
+                                       float *g_w, const float *g_sh, float *slot)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= S.N) return;
     const float gm = __uint_as_float(*gmax_bits);
     float A[kTAcc];
     for (int k = 0; k < kTAcc; ++k)
@@ -521,7 +519,7 @@ __global__ void __launch_bounds__(256) k_tfinal(SceneView S, CamParams C, const 
         if (g_scale) { g_scale[2 * i] = 0.f; g_scale[2 * i + 1] = 0.f; }
         if (g_w) g_w[i] = 0.f;
         if (g_rot) for (int a = 0; a < 4; ++a) g_rot[4 * i + a] = 0.f;
-        if (g_sh) store_zeros(g_sh + 3 * K * i, 3 * K);
+        if (g_sh) put_sh_zeros(slot);
         return;
     }
     float q[4], R[9], qn[4], qnorm;
@@ -561,7 +559,7 @@ __global__ void __launch_bounds__(256) k_tfinal(SceneView S, CamParams C, const 
     case 4: sh_weighted_grad<4>(S.s_sh, i, S.sh_dtype, gc, dir, gd); break;
     default: break;   // degree 0: the colour does not depend on the direction
     }
-    if (g_sh) store_sh_grad(g_sh + 3 * K * i, K, Y, gc, nullptr);
+    if (g_sh) put_sh_row(slot, K, Y, gc, nullptr);
     if (dist > 0.f) {
         const float pr = gd[0] * dir[0] + gd[1] * dir[1] + gd[2] * dir[2];
         for (int a = 0; a < 3; ++a) gp[a] -= (gd[a] - pr * dir[a]) / dist;
@@ -587,6 +585,18 @@ __global__ void __launch_bounds__(256) k_tfinal(SceneView S, CamParams C, const 
                    qy * GR[1][2] + qx * GR[2][0] + qy * GR[2][1]);
     const float pr = gq[0] * wq + gq[1] * qx + gq[2] * qy + gq[3] * qz;
     for (int a = 0; a < 4; ++a) g_rot[4 * i + a] = (gq[a] - pr * qn[a]) / qnorm;
+}
+__global__ void __launch_bounds__(256) k_tfinal(SceneView S, CamParams C, const float4 *__restrict__ tside,
+                                                const long long *__restrict__ acc,
+                                                const unsigned *gmax_bits, float *g_pos, float *g_rot,
+                                                float *g_scale, float *g_w, float *g_sh)
+{
+    __shared__ float slots[256 * kShSlot];
+    const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (i < S.N)
+        tfinal(S, C, i, tside, acc, gmax_bits, g_pos, g_rot, g_scale, g_w, g_sh, slots + kShSlot * threadIdx.x);
+    if (g_sh)
+        flush_sh_rows(g_sh, i & ~(int64_t)31, S.N, (S.deg + 1) * (S.deg + 1), slots + kShSlot * (threadIdx.x & ~31u));
 }
 
 // Contribution score (Eq. 9): per Gaussian, the warp sweeps its pixels; the
