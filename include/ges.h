@@ -361,7 +361,7 @@ GES_API ges_status ges_count_fragments(ges_scene *scene, const ges_camera *cam, 
  * render is launched once for all views: the preprocess (when a scene has
  * several views, first a colour pass that evaluates Eq. 1 for all of them
  * from one read of each SH row; then one set-up launch per primitive kind),
- * the scans, the fill and the raster.  The raster is persistent and hands
+ * the scan, the fill and the raster.  The raster is persistent and hands
  * out (view, tile) work items, so small and large views balance across the
  * GPU.  Per-view semantics are exactly those of ges_render_ex.
  *
