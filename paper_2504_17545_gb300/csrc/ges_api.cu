@@ -1371,10 +1371,11 @@ namespace {
 
 // ges_render_batch through a batch graph kept on the first view's scene.  The
 // key is what the graph bakes in: the views' image sizes, the scenes'
-// primitive counts, kinds and storage types, and the options.  With the same
-// key the call only rewrites the view table (cameras, outputs, attribute
-// pointers) and replays the graph; otherwise (or when the tile lists of the
-// kept graph overflow for new cameras) it builds a new one, without tuning.
+// primitive counts, kinds, storage types and SH row alignment (which chooses
+// the set-up kernel), and the options.  With the same key the call only
+// rewrites the view table (cameras, outputs, attribute pointers) and replays
+// the graph; otherwise (or when the tile lists of the kept graph overflow for
+// new cameras) it builds a new one, without tuning.
 ges_status render_batch_engine(ges_scene *const *scenes, const std::vector<CamParams> &C, const ges_camera *cams,
                                const int32_t *sov, int n, const OptParams &O, const ges_render_opts *opts,
                                float *const *out_rgb, float *const *out_depth)
@@ -1396,7 +1397,7 @@ ges_status render_batch_engine(ges_scene *const *scenes, const std::vector<CamPa
             if (T.s_pos == S.s_pos && T.g_pos == S.g_pos && T.s_sh == S.s_sh && T.g_sh == S.g_sh) { grp = w; break; }
         }
         key.insert(key.end(), {(int64_t)sov[v], (int64_t)grp, S.N, S.M, S.gdim, S.deg, S.attr_dtype, S.sh_dtype,
-                               (int64_t)(S.g_filt3 != nullptr), C[v].W, C[v].H,
+                               (int64_t)(S.g_filt3 != nullptr), (int64_t)sh_rows_aligned(S), C[v].W, C[v].H,
                                (int64_t)(out_depth && out_depth[v])});
     }
     for (int attempt = 0; attempt < 2; ++attempt) {

@@ -1526,10 +1526,9 @@ static size_t stage_smem(int T, int row_bytes)
 int staged_row_bytes(const SceneView &S, int T)
 {
     const int row = 3 * kShRows * (S.sh_dtype == GES_F32 ? 4 : 2);
-    const bool aligned = ((reinterpret_cast<uintptr_t>(S.s_sh) | reinterpret_cast<uintptr_t>(S.g_sh)) & 15) == 0;
     // two CTAs of an SM (1 KB of each is the system's, the batch's keep a view
     // entry): with one the set-up is slower than with direct loads
-    return S.deg == 3 && aligned && 2 * (stage_smem(T, row) + 2048) <= (size_t)228 * 1024 ? row : 0;
+    return S.deg == 3 && sh_rows_aligned(S) && 2 * (stage_smem(T, row) + 2048) <= (size_t)228 * 1024 ? row : 0;
 }
 
 cudaError_t prepare_forward_kernels()

@@ -168,6 +168,11 @@ size_t local_bins_smem(int T, bool fill);
 // tiles, or 0 where it does not apply: other degrees, unaligned rows, too many
 // tiles for two CTAs per SM.
 int staged_row_bytes(const SceneView &S, int T);
+// The staged set-up copies SH rows 16 bytes at a time: both arrays start there.
+inline bool sh_rows_aligned(const SceneView &S)
+{
+    return ((reinterpret_cast<uintptr_t>(S.s_sh) | reinterpret_cast<uintptr_t>(S.g_sh)) & 15) == 0;
+}
 // Binning through per-CTA histograms; otherwise with global counters.
 inline bool local_binning(const ViewScratch &X, int T) { return X.hist != nullptr && T <= kLocalMaxTiles; }
 cudaError_t prepare_forward_kernels();   // once per device: large dynamic shared memory
