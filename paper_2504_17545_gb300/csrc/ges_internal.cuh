@@ -724,7 +724,10 @@ __device__ __forceinline__ bool disc_setup(const CamParams &C, const df *P, cons
         const float D02 = M[0][1] * M[1][2] - M[0][2] * M[1][1];
         const float D12 = M[0][2] * M[1][0] - M[0][0] * M[1][2];
         const float du = D02 * D02 - D00 * D22, dv = D12 * D12 - D11 * D22;
-        if (D22 != 0.f && du >= 0.f && dv >= 0.f && isfinite(du) && isfinite(dv)) {
+        // (products of this size for discs of thousands of image widths: below
+        // it they underflow, and the box would close around the reference pixel)
+        constexpr float kTiny = 1e-36f;
+        if (D22 != 0.f && du >= kTiny && dv >= kTiny && isfinite(du) && isfinite(dv)) {
             const float sdu = sqrtf(du), sdv = sqrtf(dv);
             const float u1 = (D02 - sdu) / D22, u2 = (D02 + sdu) / D22;
             const float v1 = (D12 - sdv) / D22, v2 = (D12 + sdv) / D22;
