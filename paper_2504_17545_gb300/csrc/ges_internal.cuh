@@ -101,7 +101,8 @@ struct ViewScratch {
     // 3D Gaussians with geometry outputs (normal, centre depth), unused
     float4 *g_aux = nullptr;
     // [N][4] camera-space frame of each surfel for the translucent render:
-    // (P, s1), (U, s2), (V, -), (N, -); written when non-null
+    // (P, s1), (U, s2), (V, +-m1), (N, m2), m its moment scales (see
+    // moment_fine; negative: moment_rare); written when non-null
     float4 *s_tside = nullptr;
     // [M] Gaussian colours in 2^-16 units, written by the batch's colour pass
     // before the set-up, which copies them into the records; null elsewhere
@@ -542,6 +543,29 @@ __device__ __forceinline__ unsigned depth_key(float z)
     return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
 }
 
+// Powers of two that the translucent backward multiplies a surfel's moments by
+// before they are rounded to fixed point, and divides by afterwards.  What ends
+// divided by a scale s takes moment_fine(s) >= 2^-5 / s (1 for s >= 2^-5), what
+// ends multiplied by s moment_coarse(s) > s, the mixed moment moment_mixed(s1, s2),
+// so that no gradient gets a coarser step than max |dL/dC| 2^-24 at any scale
+// from 2^-23 to 2^23.  With none of them (steps of 2^-30 before the division)
+// surfels of scale 1e-3 had 30 times that step, and the position gradients of
+// faint ones an error of 1.3e-3 instead of 5e-5.
+__device__ __forceinline__ int float_exp(float s) { return (int)(__float_as_uint(s) >> 23 & 255u) - 127; }   // 2^e <= s < 2^(e+1)
+__device__ __forceinline__ float pow2i(int e) { return __int_as_float((127 + e) << 23); }
+__device__ __forceinline__ float moment_fine(float s) { return pow2i(min(max(-5 - float_exp(s), 0), 18)); }
+__device__ __forceinline__ float moment_coarse(float s) { return pow2i(min(max(float_exp(s) + 1, 0), 24)); }
+__device__ __forceinline__ float moment_mixed(float s1, float s2)
+{
+    return pow2i(min(max(abs(float_exp(s1) - float_exp(s2)) - 4, 0), 18));
+}
+// some factor but moment_fine is not 1
+__device__ __forceinline__ bool moment_rare(float s1, float s2)
+{
+    const int e1 = float_exp(s1), e2 = float_exp(s2);
+    return abs(e1 - e2) > 4 || max(e1, e2) >= 0;
+}
+
 __device__ __forceinline__ unsigned pack_xy(int x, int y) { return (unsigned)x | ((unsigned)y << 16); }
 
 // ---------------------------------------------------------------------------
@@ -786,7 +810,8 @@ __device__ __forceinline__ bool disc_setup(const CamParams &C, const df *P, cons
 // translation; opaque extent of Sec. 4.1).  Produces the raster record, the
 // colour (Eq. 1) and a conservative pixel bbox.
 // tside (translucent render only; null elsewhere, which removes the stores):
-// the camera-space frame (P, s1), (U, s2), (V, -), (N, -) of a visible surfel.
+// the camera-space frame and moment scales (P, s1), (U, s2), (V, +-m1), (N, m2)
+// of a visible surfel.
 // surfel_geom: everything but the colour (visible: drawn somewhere).
 __device__ __forceinline__ void surfel_geom(const SceneView &S, const CamParams &C, const OptParams &O,
                                             int64_t i, SurfelOut &o, float4 *tside = nullptr)
@@ -819,8 +844,9 @@ __device__ __forceinline__ void surfel_geom(const SceneView &S, const CamParams 
     if (tside) {
         tside[0] = make_float4(P[0].hi, P[1].hi, P[2].hi, s1);
         tside[1] = make_float4(tu[0], tu[1], tu[2], s2);
-        tside[2] = make_float4(tv[0], tv[1], tv[2], 0.f);
-        tside[3] = make_float4(n[0], n[1], n[2], 0.f);
+        const float m1 = moment_fine(s1);
+        tside[2] = make_float4(tv[0], tv[1], tv[2], moment_rare(s1, s2) ? -m1 : m1);
+        tside[3] = make_float4(n[0], n[1], n[2], moment_fine(s2));
     }
     o.rec = d.rec;
     o.x0 = d.x0; o.y0 = d.y0; o.x1 = d.x1; o.y1 = d.y1;

@@ -342,7 +342,10 @@ __global__ void __launch_bounds__(kRasterThreads, 4)
 // gradients of position, frame and scales themselves took twice the
 // instructions per pair (and 18 sums to reduce and to add instead of 14):
 // k_tbwd 323 -> 239 us at 1080p, 1M surfels, front first (at 3 CTAs per SM 274).
-// fr: the surfel's camera-space frame (P, s1), (U, s2), (V, -), (N, -).
+// Sums 4-8, 10 and 11 are scaled by the surfel's powers of two (moment_fine and
+// its kin); the ones that are not 1 for ordinary scales hide behind the sign
+// of m1, one branch that a warp takes as one.
+// fr: the surfel's camera-space frame (P, s1), (U, s2), (V, +-m1), (N, m2).
 __device__ __forceinline__ void t_terms(const float4 *fr, float a, float G, float wv, float T, float iz,
                                         const float *g, const float *cS, const float *col, float u, float v,
                                         const CamParams &C, float *out)
@@ -363,21 +366,27 @@ __device__ __forceinline__ void t_terms(const float4 *fr, float a, float G, floa
     const float Nd = f3.x * d0 + f3.y * d1 + f3.z;
     const float ra = rp * aa, rb = rp * bb;
     const float h = 2.f * (ra * Ud / f0.w + rb * Vd / f1.w) / Nd;
-    out[4] = ra;
-    out[5] = rb;
-    out[6] = ra * aa;
+    out[4] = ra * fabsf(f2.w);
+    out[5] = rb * f3.w;
+    out[6] = out[4] * aa;
     out[7] = ra * bb;
-    out[8] = rb * bb;
+    out[8] = out[5] * bb;
     out[9] = h;
     out[10] = h * aa;
     out[11] = h * bb;
+    if (f2.w < 0.f) {
+        out[7] *= moment_mixed(f0.w, f1.w);
+        out[10] *= moment_coarse(f0.w);
+        out[11] *= moment_coarse(f1.w);
+    }
     const float xn = 2.f * (X0 * f3.x + X1 * f3.y + X2 * f3.z);
     out[12] = ra * xn / f0.w;
     out[13] = rb * xn / f1.w;
 }
 
-// Sum k in units of max |dL/dC| 2^-30 (the sums of h, which grow with 1/s and
-// 1/N.d: 2^-24), as an integer (the fast conversion holds below 2^42).
+// The steps of the (scaled) sums, as integers: max |dL/dC| times 2^-30 for sums
+// 0 to 8, 2^-24 for the sums of h, which grow with 1/s and 1/N.d, and for 12
+// and 13 (the fast conversion holds below 2^42).
 __device__ __forceinline__ constexpr float t_units(int k) { return k < 9 ? 1073741824.f : 16777216.f; }
 __device__ __forceinline__ void t_add(unsigned long long *a, float x)
 {
@@ -478,7 +487,7 @@ __global__ void __launch_bounds__(kRasterThreads, 4)
                 // the warp's sums, each added by the lane that ends up holding it
                 unsigned long long *ak = reinterpret_cast<unsigned long long *>(acc + (int64_t)kTAcc * id);
                 warp_reduce_scatter<kTAcc>(terms, (int)lane, [&](int k, float tot) {
-                    t_add(ak + k, tot * (t_units(k) * scale));
+                    t_add(ak + k, tot * scale * t_units(k));
                 });
             }
         }
@@ -494,7 +503,7 @@ __global__ void __launch_bounds__(kRasterThreads, 4)
             t_terms(X.s_tside + 4 * (int64_t)myfront, a, G, w[myfront], !first_seen ? Tl : 1.f, iz, g, S, col, u, v,
                     C, terms);
             unsigned long long *ak = reinterpret_cast<unsigned long long *>(acc + (int64_t)kTAcc * myfront);
-            for (int k = 0; k < kTAcc; ++k) t_add(ak + k, terms[k] * (t_units(k) * scale));
+            for (int k = 0; k < kTAcc; ++k) t_add(ak + k, terms[k] * scale * t_units(k));
         }
     }
 }
@@ -509,7 +518,7 @@ __device__ __forceinline__ void tfinal(const SceneView &S, const CamParams &C, i
     const float gm = __uint_as_float(*gmax_bits);
     float A[kTAcc];
     for (int k = 0; k < kTAcc; ++k)
-        A[k] = gm > 0.f ? __ll2float_rn(__ldg(acc + (int64_t)kTAcc * i + k)) * (gm / t_units(k)) : 0.f;
+        A[k] = gm > 0.f ? __ll2float_rn(__ldg(acc + (int64_t)kTAcc * i + k)) * (1.f / t_units(k)) * gm : 0.f;
     const int K = (S.deg + 1) * (S.deg + 1);
     bool any = false;
     for (int k = 0; k < kTAcc; ++k) any |= A[k] != 0.f;
@@ -531,7 +540,12 @@ __device__ __forceinline__ void tfinal(const SceneView &S, const CamParams &C, i
     const float4 f3 = __ldg(tside + 4 * i + 3);
     const float U[3] = {f1.x, f1.y, f1.z}, V[3] = {f2.x, f2.y, f2.z}, Nn[3] = {f3.x, f3.y, f3.z};
     const float s1 = f0.w, s2 = f1.w;
-    const float Sa = A[4], Sb = A[5], Saa = A[6], Sab = A[7], Sbb = A[8], Sh = A[9], Sha = A[10], Shb = A[11];
+    // the reciprocals of powers of two up to 2^24 are exact
+    const auto inv = [](float m) { return __int_as_float(0x7f000000 - __float_as_int(m)); };
+    const float i1 = inv(fabsf(f2.w)), i2 = inv(f3.w);
+    const float Sa = A[4] * i1, Sb = A[5] * i2, Saa = A[6] * i1, Sbb = A[8] * i2, Sh = A[9];
+    const float Sab = A[7] * inv(moment_mixed(s1, s2));
+    const float Sha = A[10] * inv(moment_coarse(s1)), Shb = A[11] * inv(moment_coarse(s2));
     float gP[3], gU[3], gV[3], gN[3];
     for (int q = 0; q < 3; ++q) {
         gP[q] = Nn[q] * Sh - U[q] * (2.f * Sa / s1) - V[q] * (2.f * Sb / s2);
