@@ -365,7 +365,7 @@ __device__ __forceinline__ void t_terms(const float4 *fr, float a, float G, floa
     const float Ud = f1.x * d0 + f1.y * d1 + f1.z, Vd = f2.x * d0 + f2.y * d1 + f2.z;
     const float Nd = f3.x * d0 + f3.y * d1 + f3.z;
     const float ra = rp * aa, rb = rp * bb;
-    const float h = 2.f * (ra * Ud / f0.w + rb * Vd / f1.w) / Nd;
+    const float h = free_ ? 2.f * (ra * Ud / f0.w + rb * Vd / f1.w) / Nd : 0.f;   // (clamped: 0 / 0 where N.d is 0)
     out[4] = ra * fabsf(f2.w);
     out[5] = rb * f3.w;
     out[6] = out[4] * aa;
