@@ -468,7 +468,8 @@ __global__ void __launch_bounds__(1024) k_colscan(ViewScratch X, int T, LocalBin
 // block), the costly ones first in buckets of a quarter octave, so that none
 // starts when the rest is done: in the order of the tiles the SMs stood idle
 // for 17 % of a 1080p view's raster and 40 % of a 4-sample one's.  A batch:
-// the shared tiles, then the others, each longest first.
+// the shared tiles, then the others, each longest first (*any_shared: set to 1
+// when there is a shared one).
 // Long is above total / kShareSlots entries (total: of all views): such a
 // tile's warps would still be at work when all other tiles are done.  At half
 // that, ordinary views slow down (a shared block's z-buffers cull less: 1080p
@@ -477,7 +478,8 @@ __global__ void __launch_bounds__(1024) k_colscan(ViewScratch X, int T, LocalBin
 // lists (kShareMin) are not worth the merge.
 constexpr unsigned kShareMin = 256u;
 template <bool kBatch>
-__device__ __forceinline__ void order_body(const ViewScratch &X, int T, unsigned long long total, unsigned *sh)
+__device__ __forceinline__ void order_body(const ViewScratch &X, int T, unsigned long long total, unsigned *sh,
+                                           unsigned *any_shared = nullptr)
 {
     unsigned *start = sh;                     // [64]
     const unsigned share = max((unsigned)min(total / kShareSlots, 0x7fffffffull), kShareMin);
@@ -507,7 +509,10 @@ __device__ __forceinline__ void order_body(const ViewScratch &X, int T, unsigned
         }
         start[2 * threadIdx.x] = incl - a - b;
         start[2 * threadIdx.x + 1] = incl - b;
-        if (threadIdx.x == (kBatch ? 15 : 31)) X.status[ST_ITEMS] = incl;
+        if (threadIdx.x == (kBatch ? 15 : 31)) {
+            X.status[ST_ITEMS] = incl;
+            if (any_shared && incl) *any_shared = 1u;
+        }
     }
     __syncthreads();
     for (int t = threadIdx.x; t < T; t += kFillThreads) {
@@ -1240,6 +1245,20 @@ __device__ __forceinline__ int find_view(int n, int x, F base)
     return lo;
 }
 
+// The same by a warp, from view lo on: 32 views are compared at a time (two
+// dependent reads among 1024 views instead of ten).
+template <class F>
+__device__ __forceinline__ int warp_find_view(int lo, int n, int x, F base)
+{
+    int hi = n - 1;
+    while (lo < hi) {
+        const int step = (hi - lo + 31) >> 5, k = lo + ((int)lane_id() + 1) * step;
+        lo += step * __popc(__ballot_sync(0xffffffffu, k <= hi && base(k) <= x));
+        hi = min(hi, lo + step - 1);
+    }
+    return lo;
+}
+
 __device__ __forceinline__ void load_view(const BatchView *V, int v, BatchView &dst)
 {
     const int *src = reinterpret_cast<const int *>(V + v);
@@ -1374,11 +1393,14 @@ __global__ void __launch_bounds__(kFillThreads, 2) k_bfill(const BatchView *V, i
         __shared__ unsigned long long total;
         if (threadIdx.x == 0) total = 0ull;
         __syncthreads();
-        const unsigned *st = bv.X.status - (size_t)sv * ST_WORDS;
+        unsigned *st = bv.X.status - (size_t)sv * ST_WORDS;
+        unsigned long long mine = 0ull;
         for (int v = threadIdx.x; v < n; v += kFillThreads)
-            atomicAdd(&total, (unsigned long long)st[(size_t)v * ST_WORDS + ST_SPAIRS] + st[(size_t)v * ST_WORDS + ST_GPAIRS]);
+            mine += (unsigned long long)st[(size_t)v * ST_WORDS + ST_SPAIRS] + st[(size_t)v * ST_WORDS + ST_GPAIRS];
+        for (int d = 16; d > 0; d >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, d);
+        if (lane_id() == 0 && mine) atomicAdd(&total, mine);
         __syncthreads();
-        order_body<true>(bv.X, bv.T, total, cur);
+        order_body<true>(bv.X, bv.T, total, cur, st + (size_t)n * ST_WORDS + BW_SHARED);
     }
     else fill_local_body(bv.X, bv.T, bv.C.tiles_x, bv.C.tsx, bv.C.tsy, bv.B, c - bv.prep_base, cur, false);
 }
@@ -1410,34 +1432,41 @@ __global__ void __launch_bounds__(kRasterThreads, kRasterCtas) k_braster(const B
         if (lane_id() == 0 && atomicAdd(bv.X.status + ST_RETIRED, blocks) + blocks == all)
             *reinterpret_cast<unsigned long long *>(bv.X.status + ST_TDONE) = global_timer_ns();
     };
+    // the views with shared tiles, found 32 at a time (a view at a time, two
+    // dependent reads each, a batch of 1024 small views took 0.4 ms to look)
     unsigned dealt = blockIdx.x;     // the CTA's next one among the shared blocks of all views
-    for (int v = 0; v < n; ++v) {
-        const unsigned *st = V[v].X.status;
-        const unsigned shared = (st[ST_FLAGS] & (FLAG_SOVF | FLAG_GOVF)) ? 0u : st[ST_ITEMS];
-        if (shared == 0u) continue;
-        load(v);
-        const int lb = bv.C.tsx + bv.C.tsy - 5;
-        for (; dealt < shared << lb; dealt += gridDim.x) {
-            raster_block<kS, kG, false, true>(bv.X, bv.C, O, bv.rgb, bv.depth, kIds ? bv.id : nullptr,
-                                              kIds ? bv.aux : nullptr, GeoMaps{}, (int)bv.X.order[dealt >> lb],
-                                              (int)dealt & ((1 << lb) - 1), space);
-            if (warp == 0) retire(1u);
+    const unsigned *st = V[0].X.status;
+    for (int v0 = counter[BW_SHARED] ? 0 : n; v0 < n; v0 += 32) {
+        const int vl = v0 + (int)lane_id();
+        unsigned mine = 0u;
+        if (vl < n && !(st[(size_t)vl * ST_WORDS + ST_FLAGS] & (FLAG_SOVF | FLAG_GOVF))) mine = st[(size_t)vl * ST_WORDS + ST_ITEMS];
+        for (unsigned m = __ballot_sync(0xffffffffu, mine != 0u); m; m &= m - 1u) {
+            const int o = __ffs(m) - 1;
+            const unsigned shared = __shfl_sync(0xffffffffu, mine, o);
+            load(v0 + o);
+            const int lb = bv.C.tsx + bv.C.tsy - 5;
+            for (; dealt < shared << lb; dealt += gridDim.x) {
+                raster_block<kS, kG, false, true>(bv.X, bv.C, O, bv.rgb, bv.depth, kIds ? bv.id : nullptr,
+                                                  kIds ? bv.aux : nullptr, GeoMaps{}, (int)bv.X.order[dealt >> lb],
+                                                  (int)dealt & ((1 << lb) - 1), space);
+                if (warp == 0) retire(1u);
+            }
+            dealt -= shared << lb;
         }
-        dealt -= shared << lb;
     }
     int cur_v = -1;
     unsigned it = 0, flags = 0, shared = 0;
     constexpr int lo = 3;             // log2 blocks per tile
     static_assert(1 << lo == kOrderItems, "blocks per tile");
-    if (lane_id() == 0) it = atomicAdd(counter, 1u);
+    if (lane_id() == 0) it = atomicAdd(counter + BW_NEXT, 1u);
     it = __shfl_sync(0xffffffffu, it, 0);
     while ((int)(it >> lo) < total) {
         // the next item is taken now and used after this one: the atomic's
         // round trip overlaps the raster
         unsigned nxt = 0;
-        if (lane_id() == 0) nxt = atomicAdd(counter, 1u);
+        if (lane_id() == 0) nxt = atomicAdd(counter + BW_NEXT, 1u);
         if (cur_v < 0 || (int)(it >> lo) >= bv.tile_base + bv.T) {
-            cur_v = find_view(n, (int)(it >> lo), [&](int k) { return V[k].tile_base; });
+            cur_v = warp_find_view(max(cur_v, 0), n, (int)(it >> lo), [&](int k) { return V[k].tile_base; });
             load(cur_v);
             flags = bv.X.status[ST_FLAGS] & (FLAG_SOVF | FLAG_GOVF);
             shared = flags ? 0u : bv.X.status[ST_ITEMS];
@@ -1466,7 +1495,7 @@ cudaError_t launch_batch(const BatchView *d_views, const BatchPlan &P, const Opt
     auto mark = [&](int k) { if (ev) cudaEventRecordWithFlags(ev[k], st, cudaEventRecordExternal); };
     mark(0);
     {
-        unsigned long long *t0 = reinterpret_cast<unsigned long long *>(work_counter + 2);
+        unsigned long long *t0 = reinterpret_cast<unsigned long long *>(work_counter + BW_START);
         const size_t sm = local_bins_smem(P.max_T, false);
         const bool col = P.total_colour > 0;   // colours in the colour pass, not in the set-up
         if (col) {

@@ -40,6 +40,12 @@ enum : int {
     ST_ITEMS = 14,        // one view: items in the order array; batch: its tiles shared by a CTA's warps
     ST_WORDS = 16,
 };
+// words after a batch's view slots (zeroed with them before every launch)
+enum : int {
+    BW_NEXT = 0,          // raster: the next item
+    BW_START = 2,         // %globaltimer (ns, 64-bit, words 2-3) of the first CTA
+    BW_SHARED = 4,        // some view has tiles shared by a CTA's warps
+};
 enum : unsigned { FLAG_SOVF = 1u, FLAG_GOVF = 2u, FLAG_BADQ = 4u };
 
 struct CamParams {
