@@ -463,13 +463,14 @@ __global__ void __launch_bounds__(1024) k_colscan(ViewScratch X, int T, LocalBin
 
 // The raster's work items, by one CTA while the others fill.  A tile is
 // rastered by a warp per block, or, if its list (both kinds together) is long,
-// by all warps of a CTA block after block.  One view (kBatch false): an item
-// per tile, or per block of a shared tile (above bit 24 of the word 1 +
-// block), the costly ones first in buckets of a quarter octave, so that none
-// starts when the rest is done: in the order of the tiles the SMs stood idle
-// for 17 % of a 1080p view's raster and 40 % of a 4-sample one's.  A batch:
-// the shared tiles, then the others, each longest first (*any_shared: set to 1
-// when there is a shared one).
+// by all warps of a CTA block after block.  One view: an item per tile, or per
+// block of a shared tile (above bit 24 of the word 1 + block), the costly ones
+// first in buckets of a quarter octave, so that none starts when the rest is
+// done: in the order of the tiles the SMs stood idle for 17 % of a 1080p view's
+// raster and 40 % of a 4-sample one's.  A batch: the shared tiles, then the
+// others, each longest first, then those with short lists (raster_short; not
+// counted one by one: their shared counter would be every thread's).  The
+// translucent render: the tiles, longest first.
 // Long is above total / kShareSlots entries (total: of all views): such a
 // tile's warps would still be at work when all other tiles are done.  At half
 // that, ordinary views slow down (a shared block's z-buffers cull less: 1080p
@@ -477,27 +478,48 @@ __global__ void __launch_bounds__(1024) k_colscan(ViewScratch X, int T, LocalBin
 // 1.2M primitives takes 146 instead of 83 us (580 us with no sharing).  Short
 // lists (kShareMin) are not worth the merge.
 constexpr unsigned kShareMin = 256u;
-template <bool kBatch>
-__device__ __forceinline__ void order_body(const ViewScratch &X, int T, unsigned long long total, unsigned *sh,
-                                           unsigned *any_shared = nullptr)
+// at most this many entries in each of a tile's lists: raster_short's, an entry per lane
+constexpr int kShort = 32;
+__device__ __forceinline__ bool short_lists(const int2 &sr, const int2 &gr)
 {
-    unsigned *start = sh;                     // [64]
+    return max(sr.y - sr.x, gr.y - gr.x) <= kShort;
+}
+enum OrderOf : int { ORDER_VIEW, ORDER_TILES, ORDER_BATCH };
+// Returns (to all threads) the number of shared (ORDER_BATCH) and short tiles.
+template <int kOf>
+__device__ __forceinline__ uint2 order_body(const ViewScratch &X, int T, unsigned long long total, unsigned *sh)
+{
+    unsigned *start = sh;                     // [64] buckets, then the short ones
     const unsigned share = max((unsigned)min(total / kShareSlots, 0x7fffffffull), kShareMin);
-    const auto length = [&](int t) {
+    // a tile's bucket, 0..63, costly first (not one view: 0..31 shared, 32..63 not, half octaves; 64 short)
+    bool blocks = false;
+    const auto bucket = [&](int t) {
         const int2 s = X.s_rng[t], g = X.g_rng[t];
-        return (unsigned)((s.y - s.x) + (g.y - g.x));
-    };
-    // 0..63, costly first (a batch: 0..31 shared, 32..63 not, half octaves)
-    const auto bucket = [&](unsigned n) {
+        if (kOf == ORDER_BATCH && short_lists(s, g)) return 64;
+        const unsigned n = (unsigned)((s.y - s.x) + (g.y - g.x));
         const bool sh_ = n > share;
-        const unsigned b = __float_as_uint((float)(1u + (sh_ && !kBatch ? n / 8u : n)));
-        return kBatch ? (sh_ ? 31 : 63) - min((int)(b >> 22) - (127 << 1), 31) : 63 - min((int)(b >> 21) - (127 << 2), 63);
+        blocks = kOf == ORDER_VIEW && sh_;
+        const unsigned b = __float_as_uint((float)(1u + (blocks ? n / 8u : n)));
+        return kOf != ORDER_VIEW ? (sh_ ? 31 : 63) - min((int)(b >> 22) - (127 << 1), 31) : 63 - min((int)(b >> 21) - (127 << 2), 63);
     };
-    if (threadIdx.x < 64) start[threadIdx.x] = 0u;
+    // takes places in the lane's bucket (on: it has a tile)
+    const auto take = [&](bool on, int k) {
+        unsigned at = 0;
+        if (on && k < 64) at = atomicAdd(start + k, blocks ? (unsigned)kOrderItems : 1u);
+        const unsigned m = __ballot_sync(0xffffffffu, on && k == 64);
+        if (kOf == ORDER_BATCH && m) {
+            unsigned first = 0;
+            if (lane_id() == 0) first = atomicAdd(start + 64, (unsigned)__popc(m));
+            first = __shfl_sync(0xffffffffu, first, 0);
+            if (on && k == 64) at = first + __popc(m & ((1u << lane_id()) - 1u));
+        }
+        return at;
+    };
+    if (threadIdx.x < 65) start[threadIdx.x] = 0u;
     __syncthreads();
-    for (int t = threadIdx.x; t < T; t += kFillThreads) {
-        const unsigned n = length(t);
-        atomicAdd(start + bucket(n), !kBatch && n > share ? (unsigned)kOrderItems : 1u);
+    for (int t0 = 0; t0 < T; t0 += kFillThreads) {
+        const int t = t0 + (int)threadIdx.x;
+        take(t < T, t < T ? bucket(t) : 0);
     }
     __syncthreads();
     if (threadIdx.x < 32) {
@@ -509,21 +531,25 @@ __device__ __forceinline__ void order_body(const ViewScratch &X, int T, unsigned
         }
         start[2 * threadIdx.x] = incl - a - b;
         start[2 * threadIdx.x + 1] = incl - b;
-        if (threadIdx.x == (kBatch ? 15 : 31)) {
-            X.status[ST_ITEMS] = incl;
-            if (any_shared && incl) *any_shared = 1u;
+        if (threadIdx.x == 15) start[65] = incl;
+        if (threadIdx.x == 31) {
+            start[66] = start[64];
+            start[64] = incl;
+            if (kOf == ORDER_VIEW) X.status[ST_ITEMS] = incl;
         }
     }
     __syncthreads();
-    for (int t = threadIdx.x; t < T; t += kFillThreads) {
-        const unsigned n = length(t);
-        const bool blocks = !kBatch && n > share;
-        const unsigned at = atomicAdd(start + bucket(n), blocks ? (unsigned)kOrderItems : 1u);
+    const uint2 counts = make_uint2(start[65], start[66]);
+    for (int t0 = 0; t0 < T; t0 += kFillThreads) {
+        const int t = t0 + (int)threadIdx.x;
+        const unsigned at = take(t < T, t < T ? bucket(t) : 0);
+        if (t >= T) continue;
         if (blocks)
             for (unsigned k = 0; k < kOrderItems; ++k) X.order[at + k] = (unsigned)t | (k + 1u) << 24;
         else
             X.order[at] = (unsigned)t;
     }
+    return counts;
 }
 
 // sorted (translucent render): the lists hold sort keys (id, depth key)
@@ -565,8 +591,8 @@ __global__ void __launch_bounds__(kFillThreads, 2) k_fill_local(ViewScratch X, i
     if (blockIdx.x == 0) {
         // (the translucent kernels take whole tiles)
         const unsigned long long total = (unsigned long long)X.status[ST_SPAIRS] + X.status[ST_GPAIRS];
-        if (X.s_tside) order_body<true>(X, T, total, cur);
-        else order_body<false>(X, T, total, cur);
+        if (X.s_tside) order_body<ORDER_TILES>(X, T, total, cur);
+        else order_body<ORDER_VIEW>(X, T, total, cur);
     }
     else fill_local_body(X, T, tiles_x, tsx, tsy, B, blockIdx.x - 1, cur, X.s_tside != nullptr);
 }
@@ -1154,12 +1180,6 @@ __device__ __forceinline__ void tile_lists(const ViewScratch &X, const OptParams
     gr = O.mode != GES_MODE_SURFELS_ONLY ? X.g_rng[tile] : make_int2(0, 0);
 }
 
-// at most this many entries in each of a tile's lists: raster_short's, an entry per lane
-constexpr int kShort = 32;
-__device__ __forceinline__ bool short_lists(const int2 &sr, const int2 &gr)
-{
-    return max(sr.y - sr.x, gr.y - gr.x) <= kShort;
-}
 // 8x4 blocks block, block + 1, ... of a tile whose lists have at most
 // 32 entries each, by one warp: an entry per lane of both lists at once, their
 // records staged once and tested one after another; no queue and no ring.
@@ -1321,20 +1341,6 @@ __device__ __forceinline__ int find_view(int n, int x, F base)
     return lo;
 }
 
-// The same by a warp, from view lo on: 32 views are compared at a time (two
-// dependent reads among 1024 views instead of ten).
-template <class F>
-__device__ __forceinline__ int warp_find_view(int lo, int n, int x, F base)
-{
-    int hi = n - 1;
-    while (lo < hi) {
-        const int step = (hi - lo + 31) >> 5, k = lo + ((int)lane_id() + 1) * step;
-        lo += step * __popc(__ballot_sync(0xffffffffu, k <= hi && base(k) <= x));
-        hi = min(hi, lo + step - 1);
-    }
-    return lo;
-}
-
 __device__ __forceinline__ void load_view(const BatchView *V, int v, BatchView &dst)
 {
     const int *src = reinterpret_cast<const int *>(V + v);
@@ -1452,7 +1458,7 @@ __global__ void __launch_bounds__(256) k_bcolscan(const BatchView *V, int n)
     colscan_body<8>(bv.X, bv.T, bv.B, blockIdx.x - bv.colscan_base, blockIdx.y == 0, part);
 }
 
-__global__ void __launch_bounds__(kFillThreads, 2) k_bfill(const BatchView *V, int n)
+__global__ void __launch_bounds__(kFillThreads, 2) k_bfill(const BatchView *V, int n, int lb)
 {
     extern __shared__ unsigned cur[];
     __shared__ __align__(16) unsigned char bv_raw[sizeof(BatchView)];
@@ -1476,20 +1482,34 @@ __global__ void __launch_bounds__(kFillThreads, 2) k_bfill(const BatchView *V, i
         for (int d = 16; d > 0; d >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, d);
         if (lane_id() == 0 && mine) atomicAdd(&total, mine);
         __syncthreads();
-        order_body<true>(bv.X, bv.T, total, cur, st + (size_t)n * ST_WORDS + BW_SHARED);
+        const uint2 c2 = order_body<ORDER_BATCH>(bv.X, bv.T, total, cur);
+        if (threadIdx.x == 0) {
+            // lists that overflowed: all tiles are counted, none is drawn
+            const bool skip = bv.X.status[ST_FLAGS] & (FLAG_SOVF | FLAG_GOVF);
+            const unsigned shared = skip ? 0u : c2.x, few = skip ? (unsigned)bv.T : c2.y;
+            bv.X.status[ST_ITEMS] = shared | few << 16;
+            bv.X.status[ST_LEFT] = batch_items(bv.T, shared, few, lb);
+            if (shared) st[(size_t)n * ST_WORDS + BW_SHARED] = 1u;
+        }
     }
     else fill_local_body(bv.X, bv.T, bv.C.tiles_x, bv.C.tsx, bv.C.tsy, bv.B, c - bv.prep_base, cur, false);
 }
 
 // Persistent raster over the tiles of the whole batch.  First the shared tiles
-// of every view (order_body), their blocks dealt out to the CTAs; then each
-// warp takes the next block of the other tiles from a counter until none is
-// left, so uneven views balance across the GPU and no warp waits for another.
-// (A whole tile per warp is as fast in large batches, but five uneven scenes of
-// at most 1000x600 pixels take 958 us instead of 582.)
+// of every view (order_body), their blocks dealt out to the CTAs; then the other
+// tiles, by warps that wait for no other: each begins with a view (all views get
+// their share of warps, so their longest tiles start first) and takes its items
+// from the view's counter until none is left, then looks for another view that
+// has some, so uneven views balance across the GPU.
+// An item is a block of a tile (with whole tiles five uneven scenes of at most
+// 1000x600 pixels took 958 us instead of 582), or half or all of a tile of short
+// lists (1 << lb blocks), whose records the warp stages once for these blocks.  With one counter for the
+// batch, an item per block everywhere and every block counted at its view by an
+// atomic that the warp waited for, batches of sparse views were bound by these:
+// eight 1080p views of 126k primitives 650 us.
 template <int kS, int kG, bool kIds>
 __global__ void __launch_bounds__(kRasterThreads, kRasterCtas) k_braster(const BatchView *V, int n, OptParams O,
-                                                                        unsigned *counter, int total)
+                                                                        const unsigned *bw, int lb)
 {
     __shared__ WarpSpace<kS, kG, false> space[kRasterWarps];
     __shared__ __align__(16) unsigned char bv_raw[kRasterWarps][sizeof(BatchView)];
@@ -1505,85 +1525,97 @@ __global__ void __launch_bounds__(kRasterThreads, kRasterCtas) k_braster(const B
     // per-view completion time: whoever finishes the view's last blocks stamps it
     const auto retire = [&](unsigned blocks) {
         const unsigned all = (unsigned)bv.T << (bv.C.tsx + bv.C.tsy - 5);
-        if (lane_id() == 0 && atomicAdd(bv.X.status + ST_RETIRED, blocks) + blocks == all)
+        if (lane_id() == 0 && blocks && atomicAdd(bv.X.status + ST_RETIRED, blocks) + blocks == all)
             *reinterpret_cast<unsigned long long *>(bv.X.status + ST_TDONE) = global_timer_ns();
     };
     // the views with shared tiles, found 32 at a time (a view at a time, two
     // dependent reads each, a batch of 1024 small views took 0.4 ms to look)
     unsigned dealt = blockIdx.x;     // the CTA's next one among the shared blocks of all views
-    const unsigned *st = V[0].X.status;
-    for (int v0 = counter[BW_SHARED] ? 0 : n; v0 < n; v0 += 32) {
+    const unsigned *st = V[0].X.status;      // (the views' status words lie together)
+    for (int v0 = bw[BW_SHARED] ? 0 : n; v0 < n; v0 += 32) {
         const int vl = v0 + (int)lane_id();
         unsigned mine = 0u;
-        if (vl < n && !(st[(size_t)vl * ST_WORDS + ST_FLAGS] & (FLAG_SOVF | FLAG_GOVF))) mine = st[(size_t)vl * ST_WORDS + ST_ITEMS];
+        if (vl < n) mine = st[(size_t)vl * ST_WORDS + ST_ITEMS] & 0xffffu;
         for (unsigned m = __ballot_sync(0xffffffffu, mine != 0u); m; m &= m - 1u) {
             const int o = __ffs(m) - 1;
-            const unsigned shared = __shfl_sync(0xffffffffu, mine, o);
-            load(v0 + o);
-            const int lb = bv.C.tsx + bv.C.tsy - 5;
-            for (; dealt < shared << lb; dealt += gridDim.x) {
-                const int tile = (int)bv.X.order[dealt >> lb];
+            const unsigned shared = __shfl_sync(0xffffffffu, mine, o) * kOrderItems;
+            if (dealt < shared) load(v0 + o);
+            for (; dealt < shared; dealt += gridDim.x) {
+                const int tile = (int)bv.X.order[dealt / kOrderItems];
                 int2 sr, gr;
                 tile_lists(bv.X, O, tile, sr, gr);
                 raster_block<kS, kG, false, true>(bv.X, bv.C, O, bv.rgb, bv.depth, kIds ? bv.id : nullptr,
-                                                  kIds ? bv.aux : nullptr, GeoMaps{}, tile,
-                                                  (int)dealt & ((1 << lb) - 1), sr, gr, space);
+                                                  kIds ? bv.aux : nullptr, GeoMaps{}, tile, (int)(dealt % kOrderItems),
+                                                  sr, gr, space);
                 if (warp == 0) retire(1u);
             }
-            dealt -= shared << lb;
+            dealt -= shared;
         }
     }
-    int cur_v = -1;
-    unsigned it = 0, flags = 0, shared = 0;
-    constexpr int lo = 3;             // log2 blocks per tile
-    static_assert(1 << lo == kOrderItems, "blocks per tile");
-    if (lane_id() == 0) it = atomicAdd(counter + BW_NEXT, 1u);
-    it = __shfl_sync(0xffffffffu, it, 0);
-    while ((int)(it >> lo) < total) {
-        // the next item is taken now and used after this one: the atomic's
-        // round trip overlaps the raster
-        unsigned nxt = 0;
-        if (lane_id() == 0) nxt = atomicAdd(counter + BW_NEXT, 1u);
-        if (cur_v < 0 || (int)(it >> lo) >= bv.tile_base + bv.T) {
-            cur_v = warp_find_view(max(cur_v, 0), n, (int)(it >> lo), [&](int k) { return V[k].tile_base; });
-            load(cur_v);
-            flags = bv.X.status[ST_FLAGS] & (FLAG_SOVF | FLAG_GOVF);
-            shared = flags ? 0u : bv.X.status[ST_ITEMS];
-        }
-        const unsigned k = (it >> lo) - (unsigned)bv.tile_base;
-        if (k >= shared) {
-            if (!flags) {
-                const int tile = (int)bv.X.order[k], block = (int)(it & (kOrderItems - 1u));
+    const int gid = (int)(blockIdx.x * kRasterWarps + warp);
+    int v = (int)((int64_t)gid * n / (gridDim.x * kRasterWarps));
+    while (v >= 0) {
+        load(v);
+        const bool skip = bv.X.status[ST_FLAGS] & (FLAG_SOVF | FLAG_GOVF);
+        const unsigned w = bv.X.status[ST_ITEMS], shared = w & 0xffffu, few = w >> 16;
+        const int items = batch_items(bv.T, shared, few, lb);
+        int *left = reinterpret_cast<int *>(bv.X.status + ST_LEFT);
+        unsigned done = 0;
+        int at = 0;
+        if (lane_id() == 0) at = atomicSub(left, 1);
+        at = __shfl_sync(0xffffffffu, at, 0);
+        while (at > 0) {
+            // the next item is taken now and used after this one: the atomic's
+            // round trip overlaps the raster
+            int nxt = 0;
+            if (lane_id() == 0) nxt = atomicSub(left, 1);
+            // a block of a longer tile, or 1 << lb blocks of a short one
+            const unsigned i = (unsigned)(items - at), cut = (bv.T - shared - few) * kOrderItems;
+            const bool brief = i >= cut;
+            done += brief ? 1u << lb : 1u;
+            const unsigned blk = brief ? cut + ((i - cut) << lb) : i;
+            if (!skip) {
+                const int tile = (int)bv.X.order[shared + blk / kOrderItems], block = (int)(blk % kOrderItems);
                 int32_t *const id = kIds ? bv.id : nullptr;
                 float *const aux = kIds ? bv.aux : nullptr;
                 int2 sr, gr;
                 tile_lists(bv.X, O, tile, sr, gr);
-                if (short_lists(sr, gr))
-                    raster_short<kS, kG, false>(bv.X, bv.C, O, bv.rgb, bv.depth, id, aux, GeoMaps{}, tile, block, 1,
-                                                sr, gr, space[warp]);
+                if (brief)
+                    raster_short<kS, kG, false>(bv.X, bv.C, O, bv.rgb, bv.depth, id, aux, GeoMaps{}, tile, block,
+                                                1 << lb, sr, gr, space[warp]);
                 else
                     raster_block<kS, kG, false, false>(bv.X, bv.C, O, bv.rgb, bv.depth, id, aux, GeoMaps{}, tile,
                                                        block, sr, gr, space);
             }
-            retire(1u);
+            at = __shfl_sync(0xffffffffu, nxt, 0);
         }
-        it = __shfl_sync(0xffffffffu, nxt, 0);
+        retire(done);
+        // another view with items left (each warp begins to look elsewhere)
+        const int from = (int)((unsigned)(v + 1 + (gid & 31)) % (unsigned)n);
+        v = -1;
+        for (int r = 0; r < n && v < 0; r += 32) {
+            const int k = r + (int)lane_id();
+            int u = from + k;
+            if (u >= n) u -= n;
+            const bool has = k < n && (int)__ldcg(st + (size_t)u * ST_WORDS + ST_LEFT) > 0;
+            const unsigned m = __ballot_sync(0xffffffffu, has);
+            if (m) v = __shfl_sync(0xffffffffu, u, __ffs(m) - 1);
+        }
     }
 }
-
 
 }  // namespace
 
 static size_t stage_smem(int T, int row_bytes);
 
-cudaError_t launch_batch(const BatchView *d_views, const BatchPlan &P, const OptParams &O, unsigned *work_counter,
+cudaError_t launch_batch(const BatchView *d_views, const BatchPlan &P, const OptParams &O, unsigned *batch_words,
                          cudaStream_t st, cudaEvent_t *ev, bool ids)
 {
     // ev (7 events or null): recorded as graph event nodes when captured
     auto mark = [&](int k) { if (ev) cudaEventRecordWithFlags(ev[k], st, cudaEventRecordExternal); };
     mark(0);
     {
-        unsigned long long *t0 = reinterpret_cast<unsigned long long *>(work_counter + BW_START);
+        unsigned long long *t0 = reinterpret_cast<unsigned long long *>(batch_words + BW_START);
         const size_t sm = local_bins_smem(P.max_T, false);
         const bool col = P.total_colour > 0;   // colours in the colour pass, not in the set-up
         if (col) {
@@ -1611,12 +1643,12 @@ cudaError_t launch_batch(const BatchView *d_views, const BatchPlan &P, const Opt
     mark(1);
     k_bcolscan<<<dim3(P.total_colscan, 2), 256, 0, st>>>(d_views, P.n);
     mark(2);
-    k_bfill<<<P.n + P.total_prep, kFillThreads, local_bins_smem(P.max_T, true), st>>>(d_views, P.n);
+    k_bfill<<<P.n + P.total_prep, kFillThreads, local_bins_smem(P.max_T, true), st>>>(d_views, P.n, P.lb);
     mark(3);
     // P.gdim: the Gaussian kind shared by all scenes of the batch
     const unsigned grid = P.raster_ctas;
     const int kind = (O.samples == 4 ? 2 : 0) + (P.gdim == 2 ? 1 : 0);
-    auto go = [&](auto kern) { kern<<<grid, kRasterThreads, 0, st>>>(d_views, P.n, O, work_counter, P.total_tiles); };
+    auto go = [&](auto kern) { kern<<<grid, kRasterThreads, 0, st>>>(d_views, P.n, O, batch_words, P.lb); };
     switch (kind + (ids ? 4 : 0)) {
     case 0: go(k_braster<1, 3, false>); break;
     case 1: go(k_braster<1, 2, false>); break;
@@ -1631,8 +1663,8 @@ cudaError_t launch_batch(const BatchView *d_views, const BatchPlan &P, const Opt
     return cudaGetLastError();
 }
 
-// (the fill's order CTA needs 64 words)
-size_t local_bins_smem(int T, bool fill) { return fill ? (size_t)(T > 64 ? T : 64) * 4 : (size_t)((T + 1) / 2) * 4; }
+// (the fill's order CTA needs 67 words)
+size_t local_bins_smem(int T, bool fill) { return fill ? (size_t)(T > 67 ? T : 67) * 4 : (size_t)((T + 1) / 2) * 4; }
 
 // Shared memory of the set-up with staged SH rows.
 static size_t stage_smem(int T, int row_bytes)

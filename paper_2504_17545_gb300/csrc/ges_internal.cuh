@@ -37,12 +37,13 @@ enum : int {
     ST_TDONE = 8,         // batch raster: %globaltimer (ns, 64-bit, words 8-9) when the last one finished
     ST_SCUR = 10,         // tile-list space handed out, surfels (64-bit, words 10-11)
     ST_GCUR = 12,         // the same for the Gaussians (words 12-13)
-    ST_ITEMS = 14,        // one view: items in the order array; batch: its tiles shared by a CTA's warps
+    ST_ITEMS = 14,        // one view: items in the order array; batch: its tiles shared by a CTA's warps,
+                          // and above bit 16 those with short lists
+    ST_LEFT = 15,         // batch raster: the view's items not yet taken (0 or less: none)
     ST_WORDS = 16,
 };
 // words after a batch's view slots (zeroed with them before every launch)
 enum : int {
-    BW_NEXT = 0,          // raster: the next item
     BW_START = 2,         // %globaltimer (ns, 64-bit, words 2-3) of the first CTA
     BW_SHARED = 4,        // some view has tiles shared by a CTA's warps
 };
@@ -124,6 +125,12 @@ constexpr int kOrderItems = 8;          // blocks of a binning tile
 constexpr int kShareSlots = 152 * kRasterCtas;   // resident raster CTAs of the GPU
 constexpr int kLocalMaxTiles = 32768;   // shared-memory cursors of the fill: 4 B per tile
 
+// raster items of a batch view's T tiles: blocks of those that are neither
+// shared nor short, and 1 << lb blocks of short ones
+__host__ __device__ constexpr int batch_items(int T, unsigned shared, unsigned few, int lb)
+{
+    return (T - (int)shared - (int)few) * kOrderItems + (int)(few * (unsigned)kOrderItems >> lb);
+}
 // One view of a batch (device table entry).  The batch kernels find their view
 // from the per-phase bases (prefix sums over the views).
 struct BatchView {
@@ -134,15 +141,16 @@ struct BatchView {
     float *rgb, *depth;
     int32_t *id;          // surfel id map [samples,H,W] or null (ges_batch_set_id_output)
     float *aux;           // W_G [H,W] or null
-    int T, tile_base, prep_base, colscan_base;
+    int T, prep_base, colscan_base;
     int sprep_base, gprep_base;   // first CTA of the view's surfel / Gaussian ranges in their own launches
 };
 struct BatchPlan {
     int n;                                   // views
-    int total_tiles, total_prep, total_colscan, max_T;
+    int total_prep, total_colscan, max_T;
     int total_sprep, total_gprep;            // preprocess CTAs of the surfel and the Gaussian launch
     int raster_ctas;                         // persistent raster grid
     int gdim;                                // Gaussian kind of every scene (2 or 3; 0 reads as 3)
+    int lb;                                  // log2 blocks of a short tile that a warp takes at a time
     int stage_bytes;                         // SH row bytes the set-up stages in shared memory; 0: direct loads
     // (view, CTA of the view) of each CTA of the surfel / Gaussian preprocess
     // launch: the views of one scene take the same primitive range one after
@@ -162,7 +170,7 @@ constexpr int kColourViews = 64;      // views whose camera centres a colour-pas
 // colour pass's start and end 5-6) or nullptr.
 // ids: the raster also writes the views' id maps and W_G where BatchView
 // points to them (a raster kernel of its own).
-cudaError_t launch_batch(const BatchView *d_views, const BatchPlan &P, const OptParams &O, unsigned *work_counter,
+cudaError_t launch_batch(const BatchView *d_views, const BatchPlan &P, const OptParams &O, unsigned *batch_words,
                          cudaStream_t st, cudaEvent_t *ev, bool ids);
 LocalBins plan_local_bins_per_cta(int64_t N, int64_t M, int64_t prims_per_cta);
 constexpr int kPrepThreads = 512;
