@@ -813,7 +813,7 @@ size_t batch_layout(ges_batch *b, const std::vector<SceneView> &S, const std::ve
 {
     size_t off = 0;
     auto take = [&](size_t bytes) { unsigned char *p = base ? base + off : nullptr; off = align256(off + bytes); return p; };
-    int prep_base = 0, col_base = 0, sprep_base = 0, gprep_base = 0;
+    int prep_base = 0, tile_base = 0, col_base = 0, sprep_base = 0, gprep_base = 0;
     for (int v = 0; v < b->n; ++v) {
         BatchView &bv = b->views[v];
         const int64_t N = std::max<int64_t>(S[v].N, 1), M = std::max<int64_t>(S[v].M, 1);
@@ -824,10 +824,12 @@ size_t batch_layout(ges_batch *b, const std::vector<SceneView> &S, const std::ve
         bv.C = C[v];
         bv.B = B;
         bv.T = T;
+        bv.tile_base = tile_base;
         bv.prep_base = prep_base;
         bv.sprep_base = sprep_base;
         bv.gprep_base = gprep_base;
         bv.colscan_base = col_base;
+        tile_base += T;
         prep_base += B.Ps + B.Pg;
         sprep_base += B.Ps;
         gprep_base += B.Pg;
@@ -1138,19 +1140,21 @@ static ges_status batch_create(ges_scene *const *scenes, const ges_camera *cams,
             P.n = n_views;
             P.raster_ctas = sms * per_sm;
             P.gdim = S[0].gdim;
-            int64_t tiles = 0;
             for (int v = 0; v < n_views; ++v) {
                 P.total_prep += b->views[v].B.Ps + b->views[v].B.Pg;
                 P.total_sprep += b->views[v].B.Ps;
                 P.total_gprep += b->views[v].B.Pg;
                 P.total_colscan += (b->views[v].T + kColTiles - 1) / kColTiles;
                 P.max_T = std::max(P.max_T, b->views[v].T);
-                tiles += b->views[v].T;
+                P.total_tiles += b->views[v].T;
             }
-            // short tiles: whole ones where a warp gets at least four tiles, halves where it gets
-            // fewer (four 859x456 views of 6k primitives: 162 us in halves, 173 whole, 181 in
-            // single blocks; eight 1080p views of 126k: 577, 553 and 675 us)
-            P.lb = tiles < (int64_t)4 * kShareSlots * kOrderItems ? 2 : 3;
+            // fewer than six blocks for each warp: one counter, blocks (see k_braster; measured on
+            // 445 to 3017 tiles, and the other way from 4140 on); else short tiles whole where a
+            // warp gets at least four tiles, in halves where it gets fewer (four 859x456 views of
+            // 6k primitives: 160 us in halves, 172 whole, 181 in blocks; eight 1080p views of
+            // 126k: 577, 553 and 675 us)
+            P.one_counter = P.total_tiles < 6 * kShareSlots;
+            P.lb = P.one_counter ? 0 : (P.total_tiles < 4 * kShareSlots * kOrderItems ? 2 : 3);
             // one set-up kernel for all views: staged rows only if every view's are
             P.stage_bytes = staged_row_bytes(S[0], P.max_T);
             for (int v = 1; v < n_views; ++v) {

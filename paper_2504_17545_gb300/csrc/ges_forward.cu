@@ -1341,6 +1341,20 @@ __device__ __forceinline__ int find_view(int n, int x, F base)
     return lo;
 }
 
+// The same by a warp, from view lo on: 32 views are compared at a time (two
+// dependent reads among 1024 views instead of ten).
+template <class F>
+__device__ __forceinline__ int warp_find_view(int lo, int n, int x, F base)
+{
+    int hi = n - 1;
+    while (lo < hi) {
+        const int step = (hi - lo + 31) >> 5, k = lo + ((int)lane_id() + 1) * step;
+        lo += step * __popc(__ballot_sync(0xffffffffu, k <= hi && base(k) <= x));
+        hi = min(hi, lo + step - 1);
+    }
+    return lo;
+}
+
 __device__ __forceinline__ void load_view(const BatchView *V, int v, BatchView &dst)
 {
     const int *src = reinterpret_cast<const int *>(V + v);
@@ -1497,19 +1511,23 @@ __global__ void __launch_bounds__(kFillThreads, 2) k_bfill(const BatchView *V, i
 
 // Persistent raster over the tiles of the whole batch.  First the shared tiles
 // of every view (order_body), their blocks dealt out to the CTAs; then the other
-// tiles, by warps that wait for no other: each begins with a view (all views get
-// their share of warps, so their longest tiles start first) and takes its items
-// from the view's counter until none is left, then looks for another view that
-// has some, so uneven views balance across the GPU.
+// tiles, by warps that wait for no other and take items until none is left, so
+// uneven views balance across the GPU.
 // An item is a block of a tile (with whole tiles five uneven scenes of at most
 // 1000x600 pixels took 958 us instead of 582), or half or all of a tile of short
-// lists (1 << lb blocks), whose records the warp stages once for these blocks.  With one counter for the
-// batch, an item per block everywhere and every block counted at its view by an
-// atomic that the warp waited for, batches of sparse views were bound by these:
-// eight 1080p views of 126k primitives 650 us.
-template <int kS, int kG, bool kIds>
+// lists (1 << lb blocks), whose records the warp stages once for these blocks.
+// Each view has a counter; a warp takes items of one view until none is left,
+// then of another.  One counter for the batch, an item per block everywhere
+// and every block counted at its view by an atomic that the warp waited for
+// bounded batches of sparse views: eight 1080p views of 126k primitives took 650
+// us, now 375, 256 views of 256x192 460 and 220, the 16-view orbit 2460 and 2400.
+// kOne: a small batch (of `tiles` tiles, a few blocks for each warp) and one
+// counter, a block per item, the views in turn: there the last long blocks decide,
+// and four uneven views of at most 750x565 pixels (1.4M primitives) take 190 us so,
+// 215 with a counter per view.
+template <int kS, int kG, bool kIds, bool kOne>
 __global__ void __launch_bounds__(kRasterThreads, kRasterCtas) k_braster(const BatchView *V, int n, OptParams O,
-                                                                        const unsigned *bw, int lb)
+                                                                        unsigned *bw, int lb, int tiles)
 {
     __shared__ WarpSpace<kS, kG, false> space[kRasterWarps];
     __shared__ __align__(16) unsigned char bv_raw[kRasterWarps][sizeof(BatchView)];
@@ -1552,54 +1570,106 @@ __global__ void __launch_bounds__(kRasterThreads, kRasterCtas) k_braster(const B
             dealt -= shared;
         }
     }
-    const int gid = (int)(blockIdx.x * kRasterWarps + warp);
-    int v = (int)((int64_t)gid * n / (gridDim.x * kRasterWarps));
-    while (v >= 0) {
-        load(v);
-        const bool skip = bv.X.status[ST_FLAGS] & (FLAG_SOVF | FLAG_GOVF);
-        const unsigned w = bv.X.status[ST_ITEMS], shared = w & 0xffffu, few = w >> 16;
-        const int items = batch_items(bv.T, shared, few, lb);
-        int *left = reinterpret_cast<int *>(bv.X.status + ST_LEFT);
-        unsigned done = 0;
-        int at = 0;
-        if (lane_id() == 0) at = atomicSub(left, 1);
+    // blocks block, block + 1, ... of tile number k of the view's order
+    const auto raster = [&](unsigned k, int block, int blocks, bool brief) {
+        const int tile = (int)bv.X.order[k];
+        int32_t *const id = kIds ? bv.id : nullptr;
+        float *const aux = kIds ? bv.aux : nullptr;
+        int2 sr, gr;
+        tile_lists(bv.X, O, tile, sr, gr);
+        if (brief)
+            raster_short<kS, kG, false>(bv.X, bv.C, O, bv.rgb, bv.depth, id, aux, GeoMaps{}, tile, block, blocks, sr,
+                                        gr, space[warp]);
+        else
+            raster_block<kS, kG, false, false>(bv.X, bv.C, O, bv.rgb, bv.depth, id, aux, GeoMaps{}, tile, block, sr,
+                                               gr, space);
+    };
+    // (the next item is always taken before this one is rastered, and used after
+    // it: the atomic's round trip overlaps the raster)
+    if constexpr (kOne) {
+        int v = -1;
+        unsigned at = 0, done = 0, shared = 0, few = 0;
+        bool skip = false;
+        if (lane_id() == 0) at = atomicAdd(bw + BW_NEXT, 1u);
         at = __shfl_sync(0xffffffffu, at, 0);
-        while (at > 0) {
-            // the next item is taken now and used after this one: the atomic's
-            // round trip overlaps the raster
-            int nxt = 0;
-            if (lane_id() == 0) nxt = atomicSub(left, 1);
-            // a block of a longer tile, or 1 << lb blocks of a short one
-            const unsigned i = (unsigned)(items - at), cut = (bv.T - shared - few) * kOrderItems;
-            const bool brief = i >= cut;
-            done += brief ? 1u << lb : 1u;
-            const unsigned blk = brief ? cut + ((i - cut) << lb) : i;
-            if (!skip) {
-                const int tile = (int)bv.X.order[shared + blk / kOrderItems], block = (int)(blk % kOrderItems);
-                int32_t *const id = kIds ? bv.id : nullptr;
-                float *const aux = kIds ? bv.aux : nullptr;
-                int2 sr, gr;
-                tile_lists(bv.X, O, tile, sr, gr);
-                if (brief)
-                    raster_short<kS, kG, false>(bv.X, bv.C, O, bv.rgb, bv.depth, id, aux, GeoMaps{}, tile, block,
-                                                1 << lb, sr, gr, space[warp]);
-                else
-                    raster_block<kS, kG, false, false>(bv.X, bv.C, O, bv.rgb, bv.depth, id, aux, GeoMaps{}, tile,
-                                                       block, sr, gr, space);
+        while (at < (unsigned)tiles * kOrderItems) {
+            unsigned nxt = 0;
+            if (lane_id() == 0) nxt = atomicAdd(bw + BW_NEXT, 1u);
+            if (v < 0 || (int)(at / kOrderItems) >= bv.tile_base + bv.T) {
+                if (v >= 0) retire(done);
+                done = 0;
+                v = warp_find_view(max(v, 0), n, (int)(at / kOrderItems), [&](int k) { return V[k].tile_base; });
+                load(v);
+                skip = bv.X.status[ST_FLAGS] & (FLAG_SOVF | FLAG_GOVF);
+                shared = bv.X.status[ST_ITEMS] & 0xffffu;
+                few = bv.X.status[ST_ITEMS] >> 16;
+            }
+            const unsigned k = at / kOrderItems - (unsigned)bv.tile_base;
+            if (k >= shared) {
+                ++done;
+                if (!skip) raster(k, (int)(at % kOrderItems), 1, k >= (unsigned)bv.T - few);
             }
             at = __shfl_sync(0xffffffffu, nxt, 0);
         }
-        retire(done);
-        // another view with items left (each warp begins to look elsewhere)
-        const int from = (int)((unsigned)(v + 1 + (gid & 31)) % (unsigned)n);
-        v = -1;
-        for (int r = 0; r < n && v < 0; r += 32) {
-            const int k = r + (int)lane_id();
-            int u = from + k;
-            if (u >= n) u -= n;
-            const bool has = k < n && (int)__ldcg(st + (size_t)u * ST_WORDS + ST_LEFT) > 0;
-            const unsigned m = __ballot_sync(0xffffffffu, has);
-            if (m) v = __shfl_sync(0xffffffffu, u, __ffs(m) - 1);
+        if (v >= 0) retire(done);
+    } else {
+        // A view with items left, by their numbers: the takers (CTAs, later warps)
+        // spread over the views as the work does (evenly, or to the next view with
+        // any items, they went from one small view to another).
+        const int windows = (n + 31) >> 5;
+        int from = (int)((uint64_t)blockIdx.x * windows / gridDim.x) * 32;     // the 32 views looked at
+        const auto pick = [&](unsigned taker, unsigned takers) {
+            for (int r = 0; r < windows; ++r) {
+                const int u = from + (int)lane_id();
+                unsigned incl = u < n ? (unsigned)max((int)__ldcg(st + (size_t)u * ST_WORDS + ST_LEFT), 0) : 0u;
+                for (int d = 1; d < 32; d <<= 1) {
+                    const unsigned y = __shfl_up_sync(0xffffffffu, incl, d);
+                    if ((int)lane_id() >= d) incl += y;
+                }
+                const unsigned all = __shfl_sync(0xffffffffu, incl, 31), k = (unsigned)((uint64_t)taker * all / takers);
+                if (all) return from + __ffs(__ballot_sync(0xffffffffu, incl > k)) - 1;
+                from = from + 32 < n ? from + 32 : 0;
+            }
+            return -1;
+        };
+        const auto take = [&](int v, int items) {
+            return atomicSub(reinterpret_cast<int *>(V[0].X.status) + (size_t)v * ST_WORDS + ST_LEFT, items);
+        };
+        // the first items are taken by the CTA, one for each warp (4864 warps that
+        // picked and took for themselves waited 10 us for the counters' lines)
+        __shared__ int first_v, first_at;
+        __syncthreads();
+        if (warp == 0) {
+            const int v = pick(blockIdx.x, gridDim.x);
+            if (lane_id() == 0) {
+                first_v = v;
+                if (v >= 0) first_at = take(v, kRasterWarps);
+            }
+        }
+        __syncthreads();
+        int v = first_v, at = first_at - (int)warp;
+        while (v >= 0) {
+            load(v);
+            const bool skip = bv.X.status[ST_FLAGS] & (FLAG_SOVF | FLAG_GOVF);
+            const unsigned w = bv.X.status[ST_ITEMS], shared = w & 0xffffu, few = w >> 16;
+            const int items = batch_items(bv.T, shared, few, lb);
+            int *left = reinterpret_cast<int *>(bv.X.status + ST_LEFT);
+            unsigned done = 0;
+            while (at > 0) {
+                int nxt = 0;
+                if (lane_id() == 0) nxt = atomicSub(left, 1);
+                // a block of a longer tile, or 1 << lb blocks of a short one
+                const unsigned i = (unsigned)(items - at), cut = (bv.T - shared - few) * kOrderItems;
+                const bool brief = i >= cut;
+                done += brief ? 1u << lb : 1u;
+                const unsigned blk = brief ? cut + ((i - cut) << lb) : i;
+                if (!skip) raster(shared + blk / kOrderItems, (int)(blk % kOrderItems), 1 << lb, brief);
+                at = __shfl_sync(0xffffffffu, nxt, 0);
+            }
+            retire(done);
+            v = pick(blockIdx.x * kRasterWarps + warp, gridDim.x * kRasterWarps);
+            if (v >= 0 && lane_id() == 0) at = take(v, 1);
+            at = __shfl_sync(0xffffffffu, at, 0);
         }
     }
 }
@@ -1648,16 +1718,19 @@ cudaError_t launch_batch(const BatchView *d_views, const BatchPlan &P, const Opt
     // P.gdim: the Gaussian kind shared by all scenes of the batch
     const unsigned grid = P.raster_ctas;
     const int kind = (O.samples == 4 ? 2 : 0) + (P.gdim == 2 ? 1 : 0);
-    auto go = [&](auto kern) { kern<<<grid, kRasterThreads, 0, st>>>(d_views, P.n, O, batch_words, P.lb); };
+    auto go = [&](auto one, auto many) {
+        if (P.one_counter) one<<<grid, kRasterThreads, 0, st>>>(d_views, P.n, O, batch_words, P.lb, P.total_tiles);
+        else many<<<grid, kRasterThreads, 0, st>>>(d_views, P.n, O, batch_words, P.lb, P.total_tiles);
+    };
     switch (kind + (ids ? 4 : 0)) {
-    case 0: go(k_braster<1, 3, false>); break;
-    case 1: go(k_braster<1, 2, false>); break;
-    case 2: go(k_braster<4, 3, false>); break;
-    case 3: go(k_braster<4, 2, false>); break;
-    case 4: go(k_braster<1, 3, true>); break;
-    case 5: go(k_braster<1, 2, true>); break;
-    case 6: go(k_braster<4, 3, true>); break;
-    default: go(k_braster<4, 2, true>); break;
+    case 0: go(k_braster<1, 3, false, true>, k_braster<1, 3, false, false>); break;
+    case 1: go(k_braster<1, 2, false, true>, k_braster<1, 2, false, false>); break;
+    case 2: go(k_braster<4, 3, false, true>, k_braster<4, 3, false, false>); break;
+    case 3: go(k_braster<4, 2, false, true>, k_braster<4, 2, false, false>); break;
+    case 4: go(k_braster<1, 3, true, true>, k_braster<1, 3, true, false>); break;
+    case 5: go(k_braster<1, 2, true, true>, k_braster<1, 2, true, false>); break;
+    case 6: go(k_braster<4, 3, true, true>, k_braster<4, 3, true, false>); break;
+    default: go(k_braster<4, 2, true, true>, k_braster<4, 2, true, false>); break;
     }
     mark(4);
     return cudaGetLastError();

@@ -44,6 +44,7 @@ enum : int {
 };
 // words after a batch's view slots (zeroed with them before every launch)
 enum : int {
+    BW_NEXT = 0,          // raster with one counter: the next item
     BW_START = 2,         // %globaltimer (ns, 64-bit, words 2-3) of the first CTA
     BW_SHARED = 4,        // some view has tiles shared by a CTA's warps
 };
@@ -141,15 +142,16 @@ struct BatchView {
     float *rgb, *depth;
     int32_t *id;          // surfel id map [samples,H,W] or null (ges_batch_set_id_output)
     float *aux;           // W_G [H,W] or null
-    int T, prep_base, colscan_base;
+    int T, tile_base, prep_base, colscan_base;
     int sprep_base, gprep_base;   // first CTA of the view's surfel / Gaussian ranges in their own launches
 };
 struct BatchPlan {
     int n;                                   // views
-    int total_prep, total_colscan, max_T;
+    int total_tiles, total_prep, total_colscan, max_T;
     int total_sprep, total_gprep;            // preprocess CTAs of the surfel and the Gaussian launch
     int raster_ctas;                         // persistent raster grid
     int gdim;                                // Gaussian kind of every scene (2 or 3; 0 reads as 3)
+    bool one_counter;                        // raster items: one counter for all views, or one for each
     int lb;                                  // log2 blocks of a short tile that a warp takes at a time
     int stage_bytes;                         // SH row bytes the set-up stages in shared memory; 0: direct loads
     // (view, CTA of the view) of each CTA of the surfel / Gaussian preprocess
