@@ -1584,34 +1584,49 @@ __global__ void __launch_bounds__(kRasterThreads, kRasterCtas) k_braster(const B
             raster_block<kS, kG, false, false>(bv.X, bv.C, O, bv.rgb, bv.depth, id, aux, GeoMaps{}, tile, block, sr,
                                                gr, space);
     };
+    // What a warp keeps of its view from item to item, in shared memory: nothing of
+    // it holds a register through the raster.
+    struct Own {
+        int v;
+        unsigned done;                  // blocks done, not yet counted at the view (lane 0's)
+        unsigned shared, few;           // the view's shared and short tiles
+        bool skip;                      // its lists overflowed
+    };
+    __shared__ Own own[kRasterWarps];
+    volatile Own &my = own[warp];
+    const auto enter = [&](int v) {
+        load(v);
+        const unsigned w = bv.X.status[ST_ITEMS];
+        my.v = v;
+        my.done = 0u;
+        my.shared = w & 0xffffu;
+        my.few = w >> 16;
+        my.skip = bv.X.status[ST_FLAGS] & (FLAG_SOVF | FLAG_GOVF);
+        __syncwarp();
+    };
     // (the next item is always taken before this one is rastered, and used after
     // it: the atomic's round trip overlaps the raster)
     if constexpr (kOne) {
-        int v = -1;
-        unsigned at = 0, done = 0, shared = 0, few = 0;
-        bool skip = false;
+        unsigned at = 0;
         if (lane_id() == 0) at = atomicAdd(bw + BW_NEXT, 1u);
         at = __shfl_sync(0xffffffffu, at, 0);
+        my.v = -1;
         while (at < (unsigned)tiles * kOrderItems) {
             unsigned nxt = 0;
             if (lane_id() == 0) nxt = atomicAdd(bw + BW_NEXT, 1u);
-            if (v < 0 || (int)(at / kOrderItems) >= bv.tile_base + bv.T) {
-                if (v >= 0) retire(done);
-                done = 0;
-                v = warp_find_view(max(v, 0), n, (int)(at / kOrderItems), [&](int k) { return V[k].tile_base; });
-                load(v);
-                skip = bv.X.status[ST_FLAGS] & (FLAG_SOVF | FLAG_GOVF);
-                shared = bv.X.status[ST_ITEMS] & 0xffffu;
-                few = bv.X.status[ST_ITEMS] >> 16;
+            if (my.v < 0 || (int)(at / kOrderItems) >= bv.tile_base + bv.T) {
+                if (my.v >= 0) retire(my.done);
+                const int v = warp_find_view(max(my.v, 0), n, (int)(at / kOrderItems), [&](int k) { return V[k].tile_base; });
+                enter(v);
             }
             const unsigned k = at / kOrderItems - (unsigned)bv.tile_base;
-            if (k >= shared) {
-                ++done;
-                if (!skip) raster(k, (int)(at % kOrderItems), 1, k >= (unsigned)bv.T - few);
+            if (k >= my.shared) {
+                if (lane_id() == 0) my.done = my.done + 1u;
+                if (!my.skip) raster(k, (int)(at % kOrderItems), 1, k >= (unsigned)bv.T - my.few);
             }
             at = __shfl_sync(0xffffffffu, nxt, 0);
         }
-        if (v >= 0) retire(done);
+        if (my.v >= 0) retire(my.done);
     } else {
         // A view with items left, by their numbers: the takers (CTAs, later warps)
         // spread over the views as the work does (evenly, or to the next view with
@@ -1649,24 +1664,20 @@ __global__ void __launch_bounds__(kRasterThreads, kRasterCtas) k_braster(const B
         __syncthreads();
         int v = first_v, at = first_at - (int)warp;
         while (v >= 0) {
-            load(v);
-            const bool skip = bv.X.status[ST_FLAGS] & (FLAG_SOVF | FLAG_GOVF);
-            const unsigned w = bv.X.status[ST_ITEMS], shared = w & 0xffffu, few = w >> 16;
-            const int items = batch_items(bv.T, shared, few, lb);
-            int *left = reinterpret_cast<int *>(bv.X.status + ST_LEFT);
-            unsigned done = 0;
+            enter(v);
             while (at > 0) {
                 int nxt = 0;
-                if (lane_id() == 0) nxt = atomicSub(left, 1);
+                if (lane_id() == 0) nxt = atomicSub(reinterpret_cast<int *>(bv.X.status + ST_LEFT), 1);
                 // a block of a longer tile, or 1 << lb blocks of a short one
-                const unsigned i = (unsigned)(items - at), cut = (bv.T - shared - few) * kOrderItems;
+                const unsigned shared = my.shared, few = my.few, cut = (bv.T - shared - few) * kOrderItems;
+                const unsigned i = (unsigned)(batch_items(bv.T, shared, few, lb) - at);
                 const bool brief = i >= cut;
-                done += brief ? 1u << lb : 1u;
+                if (lane_id() == 0) my.done = my.done + (brief ? 1u << lb : 1u);
                 const unsigned blk = brief ? cut + ((i - cut) << lb) : i;
-                if (!skip) raster(shared + blk / kOrderItems, (int)(blk % kOrderItems), 1 << lb, brief);
+                if (!my.skip) raster(shared + blk / kOrderItems, (int)(blk % kOrderItems), 1 << lb, brief);
                 at = __shfl_sync(0xffffffffu, nxt, 0);
             }
-            retire(done);
+            retire(my.done);
             v = pick(blockIdx.x * kRasterWarps + warp, gridDim.x * kRasterWarps);
             if (v >= 0 && lane_id() == 0) at = take(v, 1);
             at = __shfl_sync(0xffffffffu, at, 0);
