@@ -800,9 +800,11 @@ __host__ __device__ constexpr int few_surfels() { return kS == 4 ? 12 : 8; }
 // staged records and a pixel per lane the raster took 201 us of a 1080p view
 // (1M surfels + 300k Gaussians), 208 us of a 4-sample one; with this and the
 // tiles in order of length 139 and 143 us.
-// kRowUnroll: all four rows unrolled are 2.6 % faster in the batch's kernel and
-// 5 % slower where the Gaussian pass needs more registers.
-template <int kS, int kRowUnroll>
+// The rows are not unrolled: the raster's paths share the instruction cache, and
+// four unrolled rows (2.6 % faster when there was one path) left warps without
+// instructions 1.9 instead of 0.7 cycles per issue; the orbit batch 3740 -> 3555
+// us, a 1080p view's raster 162 -> 157, a 4K one's 663 -> 637.
+template <int kS>
 __device__ __forceinline__ void surfel_batch(const uint2 *q, float2 *slot, int n, const float4 *__restrict__ rec,
                                              const WarpBlock<kS> &B, float izn, unsigned lane, SurfelZ<kS> &z)
 {
@@ -823,7 +825,7 @@ __device__ __forceinline__ void surfel_batch(const uint2 *q, float2 *slot, int n
         const float2 ub2 = make_float2(ub, ub), gu = make_float2(a0.w, a0.w), ng = make_float2(-a0.w, -a0.w);
         const float2 au = make_float2(a1.y, a1.y), bu = make_float2(a2.x, a2.x);
         int writes = 0;
-#pragma unroll kRowUnroll
+#pragma unroll 1
         for (int r = 0; r < kRows; ++r) {
             const float dv = vb + kStep * (float)r;
             const float tz = fmaf(a1.x, dv, a0.z), ta = fmaf(a1.z, dv, a1.w), tb = fmaf(a2.y, dv, a2.z);
@@ -929,7 +931,7 @@ constexpr int kRing = 8;   // groups of list entries in flight per warp
 // touches the block and whose largest 1/z over the disc is not below every
 // 1/z the block already holds; 32 queued ones are tested as a batch.  No
 // other warp is waited for.
-template <int kS, int kRowUnroll>
+template <int kS>
 __device__ __forceinline__ void surfel_pass(ListRing<kRing> &ring, const float4 *__restrict__ rec, int n_list,
                                             const WarpBlock<kS> &B, float izn, unsigned lane, uint2 *q, float2 *slot,
                                             SurfelZ<kS> &z)
@@ -944,7 +946,7 @@ __device__ __forceinline__ void surfel_pass(ListRing<kRing> &ring, const float4 
         n += __popc(mask);
         __syncwarp();
         if (n < 32) continue;
-        surfel_batch<kS, kRowUnroll>(q, slot, 32, rec, B, izn, lane, z);
+        surfel_batch<kS>(q, slot, 32, rec, B, izn, lane, z);
         // the ones left over, against the depths found meanwhile
         const bool more = 32 + (int)lane < n;
         const uint2 l = more ? q[32 + lane] : make_uint2(0u, 0u);
@@ -954,7 +956,7 @@ __device__ __forceinline__ void surfel_pass(ListRing<kRing> &ring, const float4 
         n = __popc(lm);
         __syncwarp();
     }
-    if (n) surfel_batch<kS, kRowUnroll>(q, slot, n, rec, B, izn, lane, z);
+    if (n) surfel_batch<kS>(q, slot, n, rec, B, izn, lane, z);
     __syncwarp();
 }
 
@@ -1257,8 +1259,7 @@ __device__ __forceinline__ void raster_block(const ViewScratch &X, const CamPara
     // ---------------- pass 1: surfel z-buffer ----------------
     SurfelZ<kS> z;
     z.init(B.in_img);
-    surfel_pass<kS, kS == 1 && kG == 3 && !kGeo ? 4 : 1>(ring, X.s_rec, sr.y - sr.x - first, B, C.izn, lane, w.q,
-                                                         w.slot, z);
+    surfel_pass<kS>(ring, X.s_rec, sr.y - sr.x - first, B, C.izn, lane, w.q, w.slot, z);
     ring.open(X.g_list, gr.x + first, gr.y, step, w.ring, lane);   // on its way while pass 1 resolves
     if (kShared) {
 #pragma unroll
