@@ -1063,7 +1063,7 @@ static ges_status batch_create(ges_scene *const *scenes, const ges_camera *cams,
     {
         std::vector<std::pair<int, int>> ok;
         for (const auto &sh : shapes) {
-            bool fits = true;
+            bool fits = sh.first + sh.second == kTileBits;
             for (int v = 0; v < n_views; ++v) {
                 CamParams c = C[v];
                 set_tiles(c, sh.first, sh.second);

@@ -13,8 +13,9 @@
 //   k_fill_local  each CTA re-walks its visible segment and places every
 //                 (tile, primitive) pair with shared-memory cursors.
 //   k_raster      one warp per 8x4 pixel block: it reads its tile's list, culls
-//                 the entries by bbox and depth, copies the records of the rest
-//                 into its own shared slots and tests them.  Pass 1 keeps the
+//                 the entries by bbox and depth and tests the records of the
+//                 rest (short lists: all at once, see raster_short; long ones:
+//                 the warps of a CTA share a block).  Pass 1 keeps the
 //                 lexicographic min of (depth, surfel id); pass 2 accumulates
 //                 the depth-tested Gaussians (Eq. 2-4); the epilogue applies
 //                 Eq. 5.  Everything per pixel stays in registers.
@@ -27,7 +28,8 @@
 //
 // List order inside a tile is not fixed (shared-memory atomics), but the
 // z-buffer min is order independent and the Gaussian sums are accumulated
-// exactly in 64-bit fixed point (units of 2^-32), so the image is
+// exactly in 64-bit fixed point (alpha in units of 2^-30, its products with the
+// colours 2^-46, geometry sums 2^-32), so the image is
 // bit-identical run to run without any sort and without float atomics.
 #include <limits.h>
 
@@ -1543,7 +1545,7 @@ __global__ void __launch_bounds__(kRasterThreads, kRasterCtas) k_braster(const B
     };
     // per-view completion time: whoever finishes the view's last blocks stamps it
     const auto retire = [&](unsigned blocks) {
-        const unsigned all = (unsigned)bv.T << (bv.C.tsx + bv.C.tsy - 5);
+        const unsigned all = (unsigned)bv.T * kOrderItems;
         if (lane_id() == 0 && blocks && atomicAdd(bv.X.status + ST_RETIRED, blocks) + blocks == all)
             *reinterpret_cast<unsigned long long *>(bv.X.status + ST_TDONE) = global_timer_ns();
     };

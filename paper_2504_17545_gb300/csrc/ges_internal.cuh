@@ -20,9 +20,11 @@ constexpr int kTileShift = 4;           // log2 kTile
 constexpr int kRasterThreads = 256;     // 8 warps
 constexpr int kRasterCtas = 4;          // resident raster CTAs per SM (64 registers per thread)
 constexpr int kWarpW = 8, kWarpH = 4;
-// A binning tile is 2^tsx x 2^tsy pixels, tsx >= 3 and tsy >= 2: whole 8x4
-// blocks, at most kMaskBits block columns and rows together.
-constexpr int kMaskBits = 12;
+// A binning tile is 2^tsx x 2^tsy pixels, tsx >= 3, tsy >= 2 and tsx + tsy =
+// kTileBits: kOrderItems whole 8x4 blocks (the raster's items and the lists'
+// block bits count on it).
+constexpr int kTileBits = 8;
+constexpr int kOrderItems = 1 << (kTileBits - 5);   // blocks of a binning tile
 
 // status word layout (uint32 words)
 enum : int {
@@ -92,7 +94,7 @@ struct ViewScratch {
     int *s_vis, *g_vis;
     int *s_cnt, *g_cnt;   // [T]     per-tile counts (atomic binning; zero between renders)
     int2 *s_rng, *g_rng;  // [T]     (start, end) of each tile's list
-    uint2 *s_list, *g_list; // tile lists: (id, cull word), see list_word
+    uint2 *s_list, *g_list; // tile lists: (id, cull word), see surfel_key_bits
     int64_t s_cap, g_cap; // list capacities (entries)
     unsigned *status;     // [ST_WORDS]
     // local binning (per-CTA primitive ranges with shared-memory histograms);
@@ -122,7 +124,6 @@ struct LocalBins {
     int Ps, Pg;           // CTAs over surfels, over Gaussians
     int64_t Rs, Rg;       // primitives per CTA
 };
-constexpr int kOrderItems = 8;          // blocks of a binning tile
 constexpr int kShareSlots = 152 * kRasterCtas;   // resident raster CTAs of the GPU
 constexpr int kLocalMaxTiles = 32768;   // shared-memory cursors of the fill: 4 B per tile
 
