@@ -495,8 +495,8 @@ __device__ __forceinline__ uint2 order_body(const ViewScratch &X, int T, unsigne
     const unsigned share = max((unsigned)min(total / kShareSlots, 0x7fffffffull), kShareMin);
     // a tile's bucket, 0..63, costly first (not one view: 0..31 shared, 32..63 not, half octaves; 64 short)
     bool blocks = false;
-    const auto bucket = [&](int t) {
-        const int2 s = X.s_rng[t], g = X.g_rng[t];
+    const auto bucket = [&](const int2 &s, const int2 &g) {
+        blocks = false;
         if (kOf == ORDER_BATCH && short_lists(s, g)) return 64;
         const unsigned n = (unsigned)((s.y - s.x) + (g.y - g.x));
         const bool sh_ = n > share;
@@ -504,14 +504,31 @@ __device__ __forceinline__ uint2 order_body(const ViewScratch &X, int T, unsigne
         const unsigned b = __float_as_uint((float)(1u + (blocks ? n / 8u : n)));
         return kOf != ORDER_VIEW ? (sh_ ? 31 : 63) - min((int)(b >> 22) - (127 << 1), 31) : 63 - min((int)(b >> 21) - (127 << 2), 63);
     };
+    // f(t, tile t's lists) for all tiles, with t >= T for lanes past the end; the
+    // lists of kAhead tiles are read at once (this CTA ends last in sparse views)
+    constexpr int kAhead = 4;
+    const auto each_tile = [&](auto f) {
+        for (int t0 = 0; t0 < T; t0 += kAhead * kFillThreads) {
+            int2 sr[kAhead], gr[kAhead];
+#pragma unroll
+            for (int j = 0; j < kAhead; ++j) {
+                const int t = min(t0 + j * kFillThreads + (int)threadIdx.x, T - 1);
+                sr[j] = X.s_rng[t];
+                gr[j] = X.g_rng[t];
+            }
+#pragma unroll
+            for (int j = 0; j < kAhead; ++j)
+                if (t0 + j * kFillThreads < T) f(t0 + j * kFillThreads + (int)threadIdx.x, sr[j], gr[j]);
+        }
+    };
     // takes places in the lane's bucket (on: it has a tile)
     const auto take = [&](bool on, int k) {
         unsigned at = 0;
         if (on && k < 64) at = atomicAdd(start + k, blocks ? (unsigned)kOrderItems : 1u);
-        const unsigned m = __ballot_sync(0xffffffffu, on && k == 64);
-        if (kOf == ORDER_BATCH && m) {
+        if constexpr (kOf == ORDER_BATCH) {
+            const unsigned m = __ballot_sync(0xffffffffu, on && k == 64);
             unsigned first = 0;
-            if (lane_id() == 0) first = atomicAdd(start + 64, (unsigned)__popc(m));
+            if (lane_id() == 0 && m) first = atomicAdd(start + 64, (unsigned)__popc(m));
             first = __shfl_sync(0xffffffffu, first, 0);
             if (on && k == 64) at = first + __popc(m & ((1u << lane_id()) - 1u));
         }
@@ -519,10 +536,10 @@ __device__ __forceinline__ uint2 order_body(const ViewScratch &X, int T, unsigne
     };
     if (threadIdx.x < 65) start[threadIdx.x] = 0u;
     __syncthreads();
-    for (int t0 = 0; t0 < T; t0 += kFillThreads) {
-        const int t = t0 + (int)threadIdx.x;
-        take(t < T, t < T ? bucket(t) : 0);
-    }
+    each_tile([&](int t, const int2 &sr, const int2 &gr) {
+        const int k = bucket(sr, gr);
+        take(t < T, k);
+    });
     __syncthreads();
     if (threadIdx.x < 32) {
         const unsigned a = start[2 * threadIdx.x], b = start[2 * threadIdx.x + 1];
@@ -542,15 +559,15 @@ __device__ __forceinline__ uint2 order_body(const ViewScratch &X, int T, unsigne
     }
     __syncthreads();
     const uint2 counts = make_uint2(start[65], start[66]);
-    for (int t0 = 0; t0 < T; t0 += kFillThreads) {
-        const int t = t0 + (int)threadIdx.x;
-        const unsigned at = take(t < T, t < T ? bucket(t) : 0);
-        if (t >= T) continue;
+    each_tile([&](int t, const int2 &sr, const int2 &gr) {
+        const int b = bucket(sr, gr);
+        const unsigned at = take(t < T, b);
+        if (t >= T) return;
         if (blocks)
             for (unsigned k = 0; k < kOrderItems; ++k) X.order[at + k] = (unsigned)t | (k + 1u) << 24;
         else
             X.order[at] = (unsigned)t;
-    }
+    });
     return counts;
 }
 
